@@ -363,13 +363,15 @@ int lbm_selftest_wait(int64_t limit_ns);
  * LBM_ERR_PARAM. */
 int lbm_set_steps_done(lbm_handle* h, int64_t t);
 
-/* Step kernel and launch shape.  variant 0 or 1 (default): pulled-row
- * staging by the tensor memory accelerator (TMA), 128 columns per block;
- * 2: the same with 256 columns per block (two per thread); 64..256, a
+/* Step kernel and launch shape.  variant 0 or 1 (default): for FP32 and
+ * 16-bit storage pulled-row staging by the tensor memory accelerator (TMA),
+ * 128 columns per block; for FP64 storage tiles of nodes, one per thread.
+ * 2: TMA staging with 256 columns per block (two per thread); 64..256, a
  * multiple of 32: the register-pull kernel, each block owning variant - 2
  * columns.  rows_per_block >= 1, or 0 for the default (6 rows for FP32
- * storage, 12 otherwise, for the TMA kernel; about one wave of blocks for the
- * register-pull kernel).  rows_per_block (and the block width of the
+ * storage, 12 for 16-bit storage, for the TMA kernel; chosen from the grid for
+ * tiles; about one wave of blocks for the register-pull kernel); tiles take as
+ * many of the rows asked for as fit one.  rows_per_block (and the block width of the
  * register-pull kernel) never changes a bit of the result; different variants
  * agree to rounding (different FMA contraction).  Variant 2 is built for the
  * BGK collision with constant relaxation times only (LBM_ERR_PARAM with

@@ -32,8 +32,9 @@ struct lbm_handle {
   bool ready = false;
   bool lost = false;  // a step kernel left with copies in flight: reload the state
   Grid grid{};
-  int variant = TMA_PR_1, rows = 0;  // 1, 2: pulled-row TMA kernel; 64..256: register pull
-  int auto_rows = 0;                 // rows chosen for (variant, rows = 0); 0: not yet
+  int variant = TMA_PR_1, rows = 0;  // 1, 2: pulled-row TMA kernel; 3: tiles; 64..256: register pull
+  int auto_rows = 0;                 // rows chosen for (variant, rows); 0: not yet
+  int tile_lw = 0;                   // log2 of the tile's columns, with auto_rows (variant 3)
   cudaGraphExec_t graph[2] = {nullptr, nullptr};  // GRAPH_STEPS steps from buffer 0 / 1
   CUtensorMap maps[2][2];            // TMA descriptors [buffer][columns per thread - 1]
   double* partial = nullptr;  // reduction scratch: RED_BLOCKS x 4
@@ -386,6 +387,14 @@ int make_tensor_map(CUtensorMap* map, void* buffer, const lbm_params& p, const G
 
 namespace {
 
+// The automatic step kernel (variants 0 and 1): FP64 arithmetic bounds FP64
+// storage, so that takes the tile kernel, which does the least of it and spreads
+// it over all SMs (256^2 cavity 56 us a step with the pulled-row kernel, 34.6
+// with tiles; 4 x 33 channel 33 and 13.2).
+int default_variant(const lbm_handle* h) {
+  return h->p.precision == LBM_P_FP64 ? STEP_TILE : TMA_PR_1;
+}
+
 int create_impl(const lbm_params* p, void* stream, void* ext, int64_t ext_bytes, lbm_handle** out) {
   if (!out) return fail(nullptr, LBM_ERR_PARAM, "out is NULL");
   *out = nullptr;
@@ -457,6 +466,7 @@ int create_impl(const lbm_params* p, void* stream, void* ext, int64_t ext_bytes,
   }
   fill_grid(p, h->grid);
   h->grid.status = h->status;
+  h->variant = default_variant(h);
   for (int b = 0; b < 2; ++b) {
     for (int k = 0; k < 2; ++k) {
       rc = make_tensor_map(&h->maps[b][k], buf_ptr(h, b), h->p, h->grid, tma_box(k + 1), 6);
@@ -638,6 +648,12 @@ namespace {
 constexpr int GRAPH_STEPS = 32;
 
 int step_rows(lbm_handle* h) {
+  if (h->variant == STEP_TILE) {
+    if (h->auto_rows == 0)
+      tile_shape(h->p.nx, h->p.ny, h->p.correction != 0, std::max(1, h->num_sms), h->rows,
+                 &h->tile_lw, &h->auto_rows);
+    return h->auto_rows;
+  }
   if (h->rows <= 0 && h->auto_rows == 0)
     h->auto_rows = h->variant >= 64 ? auto_rows(h, h->variant) : tma_rows(h, h->variant);
   return h->rows > 0 ? h->rows : h->auto_rows;
@@ -658,7 +674,9 @@ cudaError_t enqueue_steps(lbm_handle* h, int64_t n, cudaStream_t stream) {
     g.t = (unsigned)h->steps;
     const CUtensorMap& map = h->maps[h->cur][npt - 1];
     cudaError_t e = cudaSuccess;
-    dispatch(h->p.precision, [&](auto* tag) {
+    if (variant == STEP_TILE)
+      e = launch_step_tile(g, h->tile_lw, rows, stream);
+    else dispatch(h->p.precision, [&](auto* tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
       if (variant >= 64) {
         const size_t smem = 3 * (size_t)variant * sizeof(typename Io<S>::C);
@@ -935,7 +953,7 @@ int lbm_set_launch(lbm_handle* h, int32_t variant, int32_t rows_per_block) {
   if (variant == TMA_PR_2 && (h->p.collision == LBM_COLL_MRT || h->p.mu_law != LBM_MU_TAU))
     return fail(h, LBM_ERR_PARAM,
                 "variant 2 (two nodes per thread) is built for BGK with constant tau only");
-  h->variant = variant == 0 ? TMA_PR_1 : variant;
+  h->variant = variant <= 1 ? default_variant(h) : variant;
   h->rows = rows_per_block;
   h->auto_rows = 0;
   drop_step_graphs(h);

@@ -30,6 +30,14 @@ cudaError_t launch_step_tma(const Grid& g, const CUtensorMap& map, int variant, 
 template <class S>
 int occupancy_step_tma(const Grid& g, int variant);
 
+// Tile step kernel (lbm_tile.cuh): FP64 storage, the automatic choice there.
+// Tiles of 2^lw columns x rows; tile_shape picks them from the grid (rows > 0:
+// that many rows, as far as they fit).  The launch also covers the open sides
+// and the walls of non-equilibrium extrapolation.
+enum { STEP_TILE = 3 };
+void tile_shape(int nx, int ny, bool corr, int sms, int rows, int* lw_out, int* rows_out);
+cudaError_t launch_step_tile(const Grid& g, int lw, int rows, cudaStream_t stream);
+
 struct BatchGrid;
 struct WorkItem;
 struct BatchCtl;

@@ -76,7 +76,8 @@ template <class S>
 cudaError_t dispatch_variant(const Grid& g, const CUtensorMap& map, int variant, int rows,
                              dim3 grid, cudaStream_t stream, int* occ) {
   if (variant == TMA_PR_2) return launch_mode<S, 2>(g, map, rows, grid, stream, occ);
-  return launch_mode<S, 1>(g, map, rows, grid, stream, occ);
+  if constexpr (sizeof(S) < 8) return launch_mode<S, 1>(g, map, rows, grid, stream, occ);
+  return cudaErrorInvalidValue;  // FP64 storage takes the tile kernel instead
 }
 
 template <class S>
