@@ -483,13 +483,11 @@ int create_impl(const lbm_params* p, void* stream, void* ext, int64_t ext_bytes,
 // Columns a block of the selected kernel owns.
 int block_cols(int variant) { return variant >= 64 ? variant - 2 : tma_cols(variant); }
 
-// Rows per block so that the step launches about one wave of blocks.
-// Rows per block of the pulled-row kernel.  Large grids keep the default
-// (6 rows, 12 for 16-bit storage; many waves of blocks); a grid that needs
-// fewer than 3 waves at the default takes the row count that minimises
-// waves x (rows + 2) (the 2: a block's fixed cost of staging its halo rows
-// and starting up, in rows), so that a mid-size grid runs in one full wave of
-// taller blocks instead of a wave and a fraction.
+// Rows per block of the TMA kernels.  Large FP32 grids keep the default (6 rows:
+// many waves of short blocks, which HBM likes); a grid that needs fewer than 3
+// waves of blocks at the default, and 16-bit storage on any grid, takes the row
+// count that minimises waves x (rows + 2) (the 2: a block's fixed cost of staging
+// its halo rows and starting up, in rows).
 int tma_rows(const lbm_handle* h, int variant) {
   const int r0 = std::min(h->p.ny, tma_default_rows(elem_size(h->p.precision)));
   const int bx = (h->p.nx + block_cols(variant) - 1) / block_cols(variant);
@@ -501,10 +499,11 @@ int tma_rows(const lbm_handle* h, int variant) {
   });
   const long long slots = (long long)std::max(occ, 1) * std::max(1, h->num_sms);
   auto waves = [&](int r) { return ((long long)bx * ((h->p.ny + r - 1) / r) + slots - 1) / slots; };
-  if (waves(r0) >= 3) return r0;
+  const bool large = waves(r0) >= 3;
+  if (large && elem_size(h->p.precision) != 2) return r0;
   int best = r0;
   long long cost = waves(r0) * (r0 + 2);
-  for (int r = 2; r <= std::min(h->p.ny, 64); ++r) {
+  for (int r = large ? 8 : 2; r <= std::min(h->p.ny, large ? 32 : 64); ++r) {
     const long long c = waves(r) * (r + 2);
     if (c < cost) {
       cost = c;

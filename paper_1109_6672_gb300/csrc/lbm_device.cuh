@@ -128,7 +128,8 @@ __host__ __device__ __forceinline__ const Phys<C>& phys(const Grid& g) {
 template <class S>
 struct Io;
 // dev: the buffer holds deviations from the rest equilibria (pref); sr: the
-// stores round stochastically (from_sr).
+// stores round stochastically (from_sr); raw: the stored value as it is, scale
+// times the quantity (to divides the scale out).
 template <>
 struct Io<double> {
   using C = double;
@@ -136,6 +137,8 @@ struct Io<double> {
   static constexpr bool sr = false;
   __device__ static double ld(const double* p) { return __ldg(p); }
   __device__ static double to(double v) { return v; }
+  static constexpr int scale = 1;
+  __device__ static double raw(double v) { return v; }
   __device__ static double from(double v) { return v; }
 };
 template <>
@@ -145,6 +148,8 @@ struct Io<float> {
   static constexpr bool sr = false;
   __device__ static float ld(const float* p) { return __ldg(p); }
   __device__ static float to(float v) { return v; }
+  static constexpr int scale = 1;
+  __device__ static float raw(float v) { return v; }
   __device__ static float from(float v) { return v; }
 };
 // 16-bit deviations.  FP16 holds 256 x the deviation (an exact scaling that
@@ -160,6 +165,8 @@ struct Io<__half> {
   static constexpr bool sr = true;
   __device__ static __half ld(const __half* p) { return __ldg(p); }
   __device__ static float to(__half v) { return __half2float(v) * (1.0f / 256.0f); }
+  static constexpr int scale = 256;
+  __device__ static float raw(__half v) { return __half2float(v); }
   __device__ static __half from(float v) { return __float2half_rn(v * 256.0f); }
   // |256 v| below the FP16 maximum 65504 (false for NaN)
   __device__ static bool in_range(float v) { return fabsf(v) < 255.875f; }
@@ -173,7 +180,7 @@ struct Io<__half> {
   __device__ static __half from_sr(float v, unsigned r) {
     return in_range(v) ? from_sr_in_range(v, r) : __float2half_rn(v * 256.0f);
   }
-  // two values in one stochastically rounding conversion (cvt.rs, sm_100
+  // two values (scaled) in one stochastically rounding conversion (cvt.rs, sm_100
   // family): the random word r supplies the bits of both (bits 28-16 the
   // first value's, 12-0 the second's).  No saturation: non-finite values
   // stay non-finite, and a finite 256 v at or above 65536 becomes infinite
@@ -181,7 +188,7 @@ struct Io<__half> {
   // diverging state is still flagged
   __device__ static void from_sr2(float va, float vb, unsigned r, __half& sa, __half& sb) {
     unsigned d;
-    asm("cvt.rs.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(va * 256.0f), "f"(vb * 256.0f), "r"(r));
+    asm("cvt.rs.f16x2.f32 %0, %1, %2, %3;" : "=r"(d) : "f"(va), "f"(vb), "r"(r));
     sa = __ushort_as_half((unsigned short)(d >> 16));
     sb = __ushort_as_half((unsigned short)(d & 0xFFFFu));
   }
@@ -193,6 +200,8 @@ struct Io<__nv_bfloat16> {
   static constexpr bool sr = true;
   __device__ static __nv_bfloat16 ld(const __nv_bfloat16* p) { return __ldg(p); }
   __device__ static float to(__nv_bfloat16 v) { return __bfloat162float(v); }
+  static constexpr int scale = 1;
+  __device__ static float raw(__nv_bfloat16 v) { return __bfloat162float(v); }
   __device__ static __nv_bfloat16 from(float v) { return __float2bfloat16_rn(v); }
   // finite (false for infinities and NaN)
   __device__ static bool in_range(float v) { return fabsf(v) <= 3.40282347e38f; }
@@ -284,6 +293,18 @@ __device__ __forceinline__ void pull(const Grid& g, const S* __restrict__ src, i
   for (int a = 0; a < NPOP; ++a) {
     const int q = a % 9;
     d[a] = Io<S>::to(Io<S>::ld(p + (plane(a) - plane(0)) * g.pitch - ey(q) * g.rp - ex(q)));
+  }
+}
+
+// The same, stored values as they are (Io::raw).
+template <class S>
+__device__ __forceinline__ void pull_raw(const Grid& g, const S* __restrict__ src, int x, int y,
+                                         typename Io<S>::C d[NPOP]) {
+  const S* p = src + slot(g, 0, x, y);
+#pragma unroll
+  for (int a = 0; a < NPOP; ++a) {
+    const int q = a % 9;
+    d[a] = Io<S>::raw(Io<S>::ld(p + (plane(a) - plane(0)) * g.pitch - ey(q) * g.rp - ex(q)));
   }
 }
 

@@ -10,13 +10,14 @@
 
 namespace lbm {
 
-// Pulled-row TMA step kernel (lbm_step_pr.cuh) with 128 (variant 1) or 256
-// (variant 2) columns per block; box width (columns) of one TMA copy.
+// TMA step kernels: the step over column pairs (lbm_pair.cuh; variant 1, FP32 and
+// 16-bit storage) with 128 columns per block, the pulled-row kernel
+// (lbm_step_pr.cuh; variant 2) with 256; box width (columns) of one TMA copy.
 enum { TMA_PR_1 = 1, TMA_PR_2 = 2 };
 constexpr int tma_npt(int variant) { return variant == TMA_PR_2 ? 2 : 1; }
 constexpr int tma_cols(int variant) { return 128 * tma_npt(variant); }
 constexpr int tma_box(int npt) { return npt == 1 ? 144 : 136; }
-// Default rows per block of the pulled-row kernel: small blocks, many waves,
+// Default rows per block of these kernels: small blocks, many waves,
 // dynamically balanced across SMs (measured on GB300 at 4096^2).
 inline int tma_default_rows(size_t elem_bytes) { return elem_bytes == 4 ? 6 : 12; }
 

@@ -121,10 +121,17 @@ __device__ __forceinline__ void to_pairs(const C d[NPOP], Pairs<C>& q) {
 
 // Moments (Eq. 35 with the force shift, Eq. 37 or the Eq. 38 form) and
 // q = -Q = rho u (theta - 1).  (r0, th, es) are rho, theta, Es for absolute
-// storage and rho - 1, theta - 1, Es - b/6 for deviation storage, formed as in
-// moments_m.  The populations may be held K times too large (K a power of
-// two; deviation storage): sh, the sum of h, and q are then K times too large
-// as well, the rest is not.
+// storage and rho - 1, theta - 1, Es - b/6 for deviation storage, there formed
+// from the sums of the stored deviations so that nothing is rounded at the scale
+// of the populations (the references' own sums are taken in FP64 on the host:
+// dref).  The balance of internal energy, rho (Es - b/6) - rho u^2 / 2, is then
+// one subtraction of two FP32 numbers, and FP32's correctly rounded subtraction
+// gives the value an FP64 subtraction rounded back to FP32 would: the exact
+// difference is an FP64 number when the exponents differ by at most 28, and
+// otherwise lies within 2^-28 of the larger operand, far from any FP32 rounding
+// tie.  The populations may be held K times too large (K a power of two;
+// deviation storage): sh, the sum of h, and q are then K times too large as
+// well, the rest is not.
 template <class C>
 struct Mom {
   C r0, ux, uy, th, es, sh;
@@ -169,6 +176,15 @@ __device__ __forceinline__ void pair_moments(const Phys<typename Scalar<C>::T>& 
   }
 }
 
+// q = -Q of the mirror ghost across a wall side: 2 rho u_w (theta_w - 1) - q (K
+// times too large, as q).
+template <class C, int K = 1>
+__device__ __forceinline__ C mirror_q(const Grid& g, int side, int comp, C rho, C th, C q) {
+  const Phys<C>& k = phys<C>(g);
+  const C thw = g.bc[side] == BC_ISO ? k.thw[side] : th;
+  return C(2 * K) * rho * k.uw[side][comp] * (thw - C(1)) - q;
+}
+
 // Relaxation rates of a node (node_rates): the constants, or with a viscosity
 // law mu(theta)/mu0 = L the rates w = 2 / (2 tau + 1), tau_f = tau_f0 L /
 // (rho theta), tau_h = tau_f r, over one common reciprocal.  Sutherland:
@@ -206,54 +222,52 @@ __device__ __forceinline__ void pair_rates(const Phys<typename Scalar<C>::T>& k,
 
 // Equilibria per pair, f^eq_a = fe + fo, f^eq_o = fe - fo (Eq. 18a), likewise
 // h^eq (Eq. 18b or the Eq. 38 form), as deviations from the rest equilibria for
-// deviation storage (the terms of equilibria_dev), with e.u and its square:
-//   f^eq: w rho [base + 9/2 eu^2 +- lin eu] per shell,
-//   h^eq: Es f^eq + w p [9 eu^2 - 3 u^2 + theta (3 e^2 - 2)/2 +- 3 eu],
+// deviation storage (the terms of equilibria_dev).  Per shell s (0: the axis
+// pairs, 1: the diagonals) they are linear in e.u and its square,
+//   fe = A + B (e.u)^2, fo = L e.u, he = HA + HB (e.u)^2, ho = HL e.u:
+//   f^eq = w rho [base + 9/2 eu^2 +- lin eu],
+//   h^eq = Es f^eq + w p [9 eu^2 - 3 u^2 + theta (3 e^2 - 2)/2 +- 3 eu],
 // all K times too large.
 template <class C>
-struct PairEq {
-  C eu[4], e2[4], fe[4], fo[4], he[4], ho[4], usq;
+struct Shells {
+  C eu[4], usq;
+  C A[2], B[2], L[2], HA[2], HB[2], HL[2];
 };
 template <class C, bool TOTAL, bool DEV, int K = 1>
-__device__ __forceinline__ void pair_equilibria(const Phys<typename Scalar<C>::T>& k, C rho,
-                                                const Mom<C>& m, PairEq<C>& q) {
+__device__ __forceinline__ void pair_shells(const Phys<typename Scalar<C>::T>& k, C rho,
+                                            const Mom<C>& m, Shells<C>& q) {
   using T = typename Scalar<C>::T;
   q.eu[0] = m.ux;
   q.eu[1] = m.uy;
   q.eu[2] = m.ux + m.uy;
   q.eu[3] = m.uy - m.ux;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) q.e2[i] = q.eu[i] * q.eu[i];
-  const C usq = q.e2[0] + q.e2[1];
+  const C usq = fma_(m.uy, m.uy, m.ux * m.ux);
   q.usq = usq;
   const C r1 = rho * C(T(K) / T(9)), r2 = rho * C(T(K) / T(36));
-  C A1, A2, lin1, lin2;
+  C lin1, lin2;
   if constexpr (DEV) {
     const C hu = C(-1.5) * usq;
-    A1 = fma_(r1, fma_(C(0.5), m.th, hu), m.r0 * C(T(K) / T(9)));
-    A2 = fma_(r2, fma_(C(2.0), m.th, hu), m.r0 * C(T(K) / T(36)));
+    q.A[0] = fma_(r1, fma_(C(0.5), m.th, hu), m.r0 * C(T(K) / T(9)));
+    q.A[1] = fma_(r2, fma_(C(2.0), m.th, hu), m.r0 * C(T(K) / T(36)));
     lin1 = fma_(C(-1.5), m.th, C(3.0));
     lin2 = fma_(C(3.0), m.th, C(3.0));
   } else {
     const C a0 = fma_(C(-1.5), usq, C(0.5));  // 1 - 3/2 u^2 + (theta - 1)/2 = a0 + theta/2
-    A1 = r1 * fma_(C(0.5), m.th, a0);
-    A2 = r2 * fma_(C(2.0), m.th, a0 + C(-1.5));
+    q.A[0] = r1 * fma_(C(0.5), m.th, a0);
+    q.A[1] = r2 * fma_(C(2.0), m.th, a0 + C(-1.5));
     lin1 = fma_(C(-1.5), m.th, C(4.5));
     lin2 = C(3.0) * m.th;
   }
-  const C B1 = C(4.5) * r1, B2 = C(4.5) * r2;
-  const C L1 = r1 * lin1, L2 = r2 * lin2;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    q.fe[i] = fma_(i < 2 ? B1 : B2, q.e2[i], i < 2 ? A1 : A2);
-    q.fo[i] = (i < 2 ? L1 : L2) * q.eu[i];
-  }
+  q.B[0] = C(4.5) * r1;
+  q.B[1] = C(4.5) * r2;
+  q.L[0] = r1 * lin1;
+  q.L[1] = r2 * lin2;
   const C Es = DEV ? m.es + C(k.b6) : m.es;
-  C PA1 = C(0.0), PA2 = C(0.0), PB1 = C(0.0), PB2 = C(0.0), PL1 = C(0.0), PL2 = C(0.0);
   if constexpr (TOTAL) {
     const C th = DEV ? m.th + C(1.0) : m.th;
     const C p1 = (rho * th) * C(T(K) / T(27)), p2 = p1 * C(0.25);  // w p
     const C hu = C(-3.0) * usq;
+    C PA1, PA2;
     if constexpr (DEV) {
       // w (Es - b/6) + w p (-3 u^2) + w (p theta - 1/3)(3 e^2 - 2)/2
       const C pt = fma_(rho * m.th, m.th + C(2.0), m.r0) * C(T(K) / T(27));
@@ -263,23 +277,19 @@ __device__ __forceinline__ void pair_equilibria(const Phys<typename Scalar<C>::T
       PA1 = p1 * fma_(C(0.5), th, hu);
       PA2 = p2 * fma_(C(2.0), th, hu);
     }
-    PB1 = C(9.0) * p1;
-    PB2 = C(9.0) * p2;
-    PL1 = C(3.0) * p1;
-    PL2 = C(3.0) * p2;
-  } else if constexpr (DEV) {
-    PA1 = m.es * C(T(K) / T(9));
-    PA2 = m.es * C(T(K) / T(36));
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    if constexpr (TOTAL) {
-      q.he[i] = fma_(Es, q.fe[i], fma_(i < 2 ? PB1 : PB2, q.e2[i], i < 2 ? PA1 : PA2));
-      q.ho[i] = fma_(Es, q.fo[i], (i < 2 ? PL1 : PL2) * q.eu[i]);
-    } else {
-      q.he[i] = DEV ? fma_(Es, q.fe[i], i < 2 ? PA1 : PA2) : Es * q.fe[i];
-      q.ho[i] = Es * q.fo[i];
-    }
+    q.HA[0] = fma_(Es, q.A[0], PA1);
+    q.HA[1] = fma_(Es, q.A[1], PA2);
+    q.HB[0] = fma_(Es, q.B[0], C(9.0) * p1);
+    q.HB[1] = fma_(Es, q.B[1], C(9.0) * p2);
+    q.HL[0] = fma_(Es, q.L[0], C(3.0) * p1);
+    q.HL[1] = fma_(Es, q.L[1], C(3.0) * p2);
+  } else {
+    q.HA[0] = DEV ? fma_(Es, q.A[0], m.es * C(T(K) / T(9))) : Es * q.A[0];
+    q.HA[1] = DEV ? fma_(Es, q.A[1], m.es * C(T(K) / T(36))) : Es * q.A[1];
+    q.HB[0] = Es * q.B[0];
+    q.HB[1] = Es * q.B[1];
+    q.HL[0] = Es * q.L[0];
+    q.HL[1] = Es * q.L[1];
   }
 }
 
@@ -305,8 +315,8 @@ __device__ __forceinline__ void pair_collide(const Phys<typename Scalar<C>::T>& 
   const C rho = DEV ? m.r0 + C(1.0) : m.r0;
   C wf, wh, kz;
   pair_rates<C, M>(k, mu_law, rho, DEV ? m.th + C(1.0) : m.th, wf, wh, kz);
-  PairEq<C> e;
-  pair_equilibria<C, MD::total, DEV, K>(k, rho, m, e);
+  Shells<C> e;
+  pair_shells<C, MD::total, DEV, K>(k, rho, m, e);
   // half of C' = C_a + F_a: even parts c[], odd parts of F_a g1 (axis y), g2
   // (diagonals); F_a = w_a [3 e.a + 9 (e.u)(e.a) - 3 u.a], a = (0, ay)
   C c[4];
@@ -330,58 +340,26 @@ __device__ __forceinline__ void pair_collide(const Phys<typename Scalar<C>::T>& 
     g1 = ay * C(T(1) / T(3));
     g2 = ay * C(T(1) / T(12));
   }
-  // twice n, even and odd parts
-  C nE[4], nO[4], fE[4], fO[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const C g = i == 1 ? g1 : g2;
-    const bool gf = MD::force && i > 0;
-    nE[i] = fma_(C(-2.0), (MD::corr || MD::force) ? e.fe[i] - c[i] : e.fe[i], q.S[i]);
-    nO[i] = fma_(C(-2.0), gf ? e.fo[i] - g : e.fo[i], q.D[i]);
-    fE[i] = (MD::corr || MD::force) ? e.fe[i] + c[i] : e.fe[i];
-    fO[i] = gf ? e.fo[i] + g : e.fo[i];
-  }
-  if constexpr (!MD::mrt) {
-    const C w1 = fma_(C(-0.5), wf, C(0.5));
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      fE[i] = fma_(w1, nE[i], fE[i]);
-      fO[i] = fma_(w1, nO[i], fO[i]);
-    }
-  } else {
-    // the even moments e, eps, pxx, pxy and the odd ones q_x, q_y of n (rows
-    // of M; n_0 from the vanishing mass), relaxed, and M^-1 of them
-    const C se = k.se > T(0) ? C(k.se) : wf, seps = k.seps > T(0) ? C(k.seps) : wf;
-    const C sq = k.sq > T(0) ? C(k.sq) : wf;
-    const C one = C(1.0);
-    const C sa = nE[0] + nE[1], sd = nE[2] + nE[3];
-    const C re = (one - se) * fma_(C(2.0), sd, sa);           // e / 3
-    const C rp = (one - seps) * fma_(C(2.0), sa, sd);         // -eps / 3
-    const C rx = (one - sq) * fma_(C(-2.0), nO[0], nO[2] - nO[3]);  // q_x
-    const C ry = (one - sq) * fma_(C(-2.0), nO[1], nO[2] + nO[3]);  // q_y
-    const C w1 = fma_(C(-0.25), wf, C(0.25));
-    const C pp = w1 * (nE[0] - nE[1]), pq = w1 * (nE[2] - nE[3]);  // pxx / 4, pxy / 4
-    const C ax = fma_(C(T(1) / T(6)), rp, re * C(T(-1) / T(12)));
-    const C dg = fma_(C(T(-1) / T(12)), rp, re * C(T(1) / T(6)));
-    const C x2 = rx * C(T(1) / T(12)), y2 = ry * C(T(1) / T(12));
-    fE[0] = fE[0] + (ax + pp);
-    fE[1] = fE[1] + (ax - pp);
-    fE[2] = fE[2] + (dg + pq);
-    fE[3] = fE[3] + (dg - pq);
-    fO[0] = fma_(C(-2.0), x2, fO[0]);
-    fO[1] = fma_(C(-2.0), y2, fO[1]);
-    fO[2] = fO[2] + (x2 + y2);
-    fO[3] = fO[3] + (y2 - x2);
-  }
-  // h relaxed, plus Eq. 36's coupling
+  // pair by pair, so that few values are live at a time: twice n (even and odd
+  // parts), h relaxed with Eq. 36's coupling, and (BGK) f relaxed
   const C zc = MD::zfull ? C(-0.5) * e.usq : C(0.0);  // Z = e.u + zc
   const C wh1 = fma_(C(-0.5), wh, C(0.5));
+  const C wf1 = fma_(C(-0.5), wf, C(0.5));
   const C kzh = C(0.5) * kz;
+  C nE[4], nO[4], bE[4], bO[4];
   C sE = C(0.0), shE = C(0.0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int a = A[i], o = opp(A[i]);
-    const C he = e.he[i], ho = e.ho[i];
+    const int a = A[i], o = opp(A[i]), s = i >> 1;
+    const C e2 = e.eu[i] * e.eu[i];
+    const C fe = fma_(e.B[s], e2, e.A[s]), fo = e.L[s] * e.eu[i];
+    const C g = i == 1 ? g1 : g2;
+    const bool cf = MD::corr || MD::force, gf = MD::force && i > 0;
+    nE[i] = fma_(C(-2.0), cf ? fe - c[i] : fe, q.S[i]);
+    nO[i] = fma_(C(-2.0), gf ? fo - g : fo, q.D[i]);
+    bE[i] = cf ? fe + c[i] : fe;
+    bO[i] = gf ? fo + g : fo;
+    const C he = fma_(e.HB[s], e2, e.HA[s]), ho = e.HL[s] * e.eu[i];
     // h* = h^eq + (1 - w_h)(h - h^eq)
     C hE = fma_(wh1, fma_(C(-2.0), he, q.Sh[i]), he);
     C hO = fma_(wh1, fma_(C(-2.0), ho, q.Dh[i]), ho);
@@ -394,12 +372,41 @@ __device__ __forceinline__ void pair_collide(const Phys<typename Scalar<C>::T>& 
         hO = fma_(kzh, e.eu[i] * nE[i], hO);
       }
     }
-    v[a] = fE[i] + fO[i];
-    v[o] = fE[i] - fO[i];
     v[9 + a] = hE + hO;
     v[9 + o] = hE - hO;
-    sE = i == 0 ? fE[i] : sE + fE[i];
     shE = i == 0 ? hE : shE + hE;
+    if constexpr (!MD::mrt) {
+      const C fE = fma_(wf1, nE[i], bE[i]), fO = fma_(wf1, nO[i], bO[i]);
+      v[a] = fE + fO;
+      v[o] = fE - fO;
+      sE = i == 0 ? fE : sE + fE;
+    }
+  }
+  if constexpr (MD::mrt) {
+    // the even moments e, eps, pxx, pxy and the odd ones q_x, q_y of n (rows
+    // of M; n_0 from the vanishing mass), relaxed, and M^-1 of them
+    const C se = k.se > T(0) ? C(k.se) : wf, seps = k.seps > T(0) ? C(k.seps) : wf;
+    const C sq = k.sq > T(0) ? C(k.sq) : wf;
+    const C one = C(1.0);
+    const C sa = nE[0] + nE[1], sd = nE[2] + nE[3];
+    const C re = (one - se) * fma_(C(2.0), sd, sa);           // e / 3
+    const C rp = (one - seps) * fma_(C(2.0), sa, sd);         // -eps / 3
+    const C rx = (one - sq) * fma_(C(-2.0), nO[0], nO[2] - nO[3]);  // q_x
+    const C ry = (one - sq) * fma_(C(-2.0), nO[1], nO[2] + nO[3]);  // q_y
+    const C w1 = C(0.5) * wf1;
+    const C pp = w1 * (nE[0] - nE[1]), pq = w1 * (nE[2] - nE[3]);  // pxx / 4, pxy / 4
+    const C ax = fma_(C(T(1) / T(6)), rp, re * C(T(-1) / T(12)));
+    const C dg = fma_(C(T(-1) / T(12)), rp, re * C(T(1) / T(6)));
+    const C x2 = rx * C(T(1) / T(12)), y2 = ry * C(T(1) / T(12));
+    const C fE[4] = {bE[0] + (ax + pp), bE[1] + (ax - pp), bE[2] + (dg + pq), bE[3] + (dg - pq)};
+    const C fO[4] = {fma_(C(-2.0), x2, bO[0]), fma_(C(-2.0), y2, bO[1]), bO[2] + (x2 + y2),
+                     bO[3] + (y2 - x2)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      v[A[i]] = fE[i] + fO[i];
+      v[opp(A[i])] = fE[i] - fO[i];
+    }
+    sE = (fE[0] + fE[1]) + (fE[2] + fE[3]);
   }
   v[0] = fma_(C(-2.0), sE, K == 1 ? m.r0 : m.r0 * C((double)K));
   v[9] = fma_(C(-2.0), shE, m.sh);

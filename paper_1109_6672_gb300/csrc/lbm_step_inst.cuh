@@ -4,37 +4,48 @@
 
 #include "lbm_launch.h"
 #include "lbm_batch.cuh"
+#include "lbm_pair.cuh"
 #include "lbm_step_pr.cuh"
 
 #include <type_traits>
 
 namespace lbm {
 
-// Kernel pointer, block size and shared memory of one configuration.
-template <class S, int NPT, int M>
-struct Cfg {
-  static constexpr int threads = PR_THREADS;
-  static size_t smem() { return PrGeom<S, NPT>::smem_bytes(); }
-  static auto kernel() { return step_pr_kernel<S, NPT, M>; }
-};
-
+// Launch (or, with occ, resident blocks per SM) of the kernel of physics mode M:
+// NPT = 1 the step over column pairs (lbm_pair.cuh), with programmatic
+// dependent launch; 2 the pulled-row kernel with two columns per thread.
 template <class S, int NPT, int M>
 cudaError_t launch_one(const Grid& g, const CUtensorMap& map, int rows, dim3 grid,
                        cudaStream_t stream, int* occ) {
-  using K = Cfg<S, NPT, M>;
+  void (*kernel)(Grid, CUtensorMap, int);
+  int threads, smem;
+  if constexpr (NPT == 1) {
+    kernel = step_pair_kernel<S, M>;
+    threads = PAIR_THREADS;
+    smem = (int)PairGeom<S>::BYTES;
+  } else {
+    kernel = step_pr_kernel<S, NPT, M>;
+    threads = PR_THREADS;
+    smem = (int)PrGeom<S, NPT>::smem_bytes();
+  }
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(K::kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)K::smem());
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  if (occ) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, K::kernel(), K::threads,
-                                                         K::smem());
-  }
-  K::kernel()<<<grid, K::threads, K::smem(), stream>>>(g, map, rows);
-  return cudaGetLastError();
+  if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, threads, smem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = NPT == 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, g, map, rows);
 }
 
 // Calls fn(std::integral_constant<int, M>{}) for the kernel of physics mode

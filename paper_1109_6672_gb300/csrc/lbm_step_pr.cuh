@@ -1,4 +1,5 @@
-// Pulled-row TMA step kernel.
+// Pulled-row TMA step kernel: launch variant 2 (two columns a thread, 256 a
+// block) and the shares of the batched kernel.
 //
 // The population planes are stored grouped by e_y (lbm_device.cuh), so the 18
 // values that lattice row r pulls are three contiguous plane groups: the
@@ -20,7 +21,7 @@
 // sets *g.status, drains its own copies (bounded) and returns.
 #pragma once
 
-#include "lbm_step_tma.cuh"
+#include "lbm_node.cuh"
 
 namespace lbm {
 
@@ -68,7 +69,7 @@ __device__ __forceinline__ void pull_pr(const S* slot, const int co[3],
 #pragma unroll
   for (int a = 0; a < NPOP; ++a) {
     const int grp = pgroup(a), lp = plane(a) - 6 * grp;
-    d[a] = Io<S>::to(slot[grp * G::NB * G::GB + lp * G::BW + co[ex(a % 9) + 1]]);
+    d[a] = Io<S>::raw(slot[grp * G::NB * G::GB + lp * G::BW + co[ex(a % 9) + 1]]);
   }
 }
 
@@ -131,6 +132,29 @@ __device__ __forceinline__ void xrec_flush(const Grid& g, S* __restrict__ dst, i
   xedge_writes<S, XS>(g, dst, x, y, v, r[12], r[13], r[14], r[15]);
 }
 
+// The 18 stores of node (x, y) at p (node slot, population stride `pitch`);
+// v: the stored quantity, 16-bit values already scaled.
+template <class S>
+__device__ __forceinline__ void pr_store(const Grid& g, S* __restrict__ p, int pitch, int x, int y,
+                                         const typename Io<S>::C* v) {
+  if constexpr (Io<S>::sr) {
+    // stochastic rounding in hardware, two populations per conversion and
+    // one random word per pair (non-finite values pass through unchanged)
+    unsigned r = sr_hash(g, x, y);
+#pragma unroll
+    for (int a = 0; a < NPOP; a += 2) {
+      r = lcg_next(r);
+      S sa, sb;
+      Io<S>::from_sr2(v[a], v[a + 1], r, sa, sb);
+      p[plane(a) * pitch] = sa;
+      p[plane(a + 1) * pitch] = sb;
+    }
+  } else {
+#pragma unroll
+    for (int a = 0; a < NPOP; ++a) p[plane(a) * pitch] = Io<S>::from(v[a]);
+  }
+}
+
 // Initialise the ring's mbarriers (once per kernel, all threads call).
 template <class S, int NPT, int DD = 0>
 __device__ __forceinline__ void pr_init(unsigned char* smem) {
@@ -183,7 +207,8 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
   using C = typename Io<S>::C;
   using G = PrGeom<S, NPT, DD, XD>;
   using SM = PrSmem<S, NPT, DD, XD>;
-  constexpr bool DEV = Io<S>::dev;  // moments carried as deviations (moments_m)
+  constexpr bool DEV = Io<S>::dev;  // moments carried as deviations (pair_moments)
+  constexpr int K = Io<S>::scale;   // factor of the stored values
   constexpr int D = G::D, TWC = G::TWC;
   constexpr unsigned long long WAIT_NS = 2000000000ull;  // 2 s
   S* ring = SM::ring(smem);
@@ -300,14 +325,18 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
         if (how == 1)
           pull_pr<S, NPT>(slot, co[i], d);
         else
-          pull<S>(g, src, gx, nr, d);
-        moments_m<S, M>(g, d, crho[i], cux[i], cuy[i], cth[i], ces[i]);
-        // Q = rho u (1 - theta) (Eq. 48); deviation storage carries rho - 1
-        // and theta - 1 instead of rho and theta
-        const C rq = DEV ? C(1) + crho[i] : crho[i];
-        const C om = DEV ? -cth[i] : C(1) - cth[i];
-        cqx[i] = rq * cux[i] * om;
-        cqy[i] = rq * cuy[i] * om;
+          pull_raw<S>(g, src, gx, nr, d);
+        // moments and q = -Q (Eq. 48, K times too large); deviation storage
+        // carries rho - 1 and theta - 1 instead of rho and theta
+        Pairs<C> pq;
+        Mom<C> m;
+        to_pairs(d, pq);
+        pair_moments<C, M, DEV, K>(phys<C>(g), pq, m, cqx[i], cqy[i]);
+        crho[i] = m.r0;
+        cux[i] = m.ux;
+        cuy[i] = m.uy;
+        cth[i] = m.th;
+        ces[i] = m.es;
       }
     }
     C* qrow = qxs + qs * (TWC + 2);
@@ -334,16 +363,25 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
         const C rho_n = DEV ? C(1) + prho[i] : prho[i];
         const C th_n = DEV ? C(1) + pth[i] : pth[i];
         const C qxl =
-            (c > 0 || !wall_l) ? qprev[lq - 1] : ghost_q<C>(g, 0, 0, rho_n, th_n, pqx[i]);
+            (c > 0 || !wall_l) ? qprev[lq - 1] : mirror_q<C, K>(g, 0, 0, rho_n, th_n, pqx[i]);
         const C qxr = (c < nx - 1 || !wall_r) ? qprev[lq + 1]
-                                              : ghost_q<C>(g, 1, 0, rho_n, th_n, pqx[i]);
+                                              : mirror_q<C, K>(g, 1, 0, rho_n, th_n, pqx[i]);
         const C qyu =
-            (ro < ny - 1 || !wall_t) ? cqy[i] : ghost_q<C>(g, 3, 1, rho_n, th_n, pqy[i]);
+            (ro < ny - 1 || !wall_t) ? cqy[i] : mirror_q<C, K>(g, 3, 1, rho_n, th_n, pqy[i]);
         const C qyd =
-            (ro > 0 || !wall_b) ? qymm[i] : ghost_q<C>(g, 2, 1, rho_n, th_n, pqy[i]);
+            (ro > 0 || !wall_b) ? qymm[i] : mirror_q<C, K>(g, 2, 1, rho_n, th_n, pqy[i]);
+        Pairs<C> pq;
+        Mom<C> m;
+        to_pairs(d, pq);
+        m.r0 = prho[i];
+        m.ux = pux[i];
+        m.uy = puy[i];
+        m.th = pth[i];
+        m.es = pes[i];
+        m.sh = pq.h0 + ((pq.Sh[0] + pq.Sh[1]) + (pq.Sh[2] + pq.Sh[3]));
         C v[27];
-        collide_m<S, M>(g, prow + c, pitch, c, ro, d, prho[i], pux[i], puy[i], pth[i], pes[i],
-                        C(0.5) * (qxr - qxl), C(0.5) * (qyu - qyd), v);
+        pair_collide<C, M, DEV, K>(phys<C>(g), g.mu_law, pq, m, qxr - qxl, qyu - qyd, v);
+        pr_store<S>(g, prow + c, pitch, c, ro, v);
         // ghost-slot writes (from absolute values): x edges inline (one
         // thread of a warp), the edge rows (every thread of the row) through
         // the general routine
@@ -351,7 +389,12 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
         if (xedge || yedge) {
           if constexpr (DEV) {
 #pragma unroll
-            for (int a = 0; a < 27; ++a) v[a] += pref<S>(g, a < 18 ? a : a - 9);
+            for (int a = 0; a < 18; ++a) v[a] = v[a] * C(1.0 / K) + pref<S>(g, a);
+          }
+          {  // h^eq with the node's own specific energy, for the wall rules
+            C fq[9];
+            equilibria_es<C>(rho_n, pux[i], puy[i], th_n,
+                             DEV ? phys<C>(g).b6 + pes[i] : pes[i], Mode<M>::total, fq, v + 18);
           }
           // a walled x side's writes are recorded and done XREC_ROWS rows at
           // a time by a whole warp (below), so that the row barrier does not

@@ -263,29 +263,37 @@ __device__ __forceinline__ void tile_ghost(const Grid& g, const S* src, S* __res
   const C uw2 = w.ux * w.ux + w.uy * w.uy;
   w.es = kp.b6 * w.th + (MD::total ? C(0.5) * uw2 : C(0));
   w.sh = C(0);
-  PairEq<C> ef, ew;
-  pair_equilibria<C, MD::total, false>(kp, m.r0, m, ef);
-  pair_equilibria<C, MD::total, false>(kp, w.r0, w, ew);
-  // normal heat flux of F's non-equilibrium part (less the wall's viscous
-  // work), taken out on an adiabatic wall
+  Shells<C> ef, ew;
+  pair_shells<C, MD::total, false>(kp, m.r0, m, ef);
+  pair_shells<C, MD::total, false>(kp, w.r0, w, ew);
+  // F's pairs less twice its equilibria; the normal heat flux of that part of h
+  // (less the wall's viscous work) is taken out on an adiabatic wall
   C en[4], qn = C(0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
+    const int s = i >> 1;
+    const C e2 = ef.eu[i] * ef.eu[i];
+    q.S[i] -= C(2) * (ef.A[s] + ef.B[s] * e2);
+    q.D[i] -= C(2) * (ef.L[s] * ef.eu[i]);
+    q.Sh[i] -= C(2) * (ef.HA[s] + ef.HB[s] * e2);
+    q.Dh[i] -= C(2) * (ef.HL[s] * ef.eu[i]);
     en[i] = C(ex(A[i]) * nxo + ey(A[i]) * nyo);
-    C hn = q.Dh[i] - C(2) * ef.ho[i];
+    C hn = q.Dh[i];
     if constexpr (MD::total) {
       const C zw2 = MD::zfull ? C(0.5) * uw2 : C(0);
-      hn -= ew.eu[i] * (q.S[i] - C(2) * ef.fe[i]) - zw2 * (q.D[i] - C(2) * ef.fo[i]);
+      hn -= ew.eu[i] * q.S[i] - zw2 * q.D[i];
     }
     qn += en[i] * hn;
   }
   if (!adia) qn = C(0);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    q.S[i] += C(2) * (ew.fe[i] - ef.fe[i]);
-    q.D[i] += C(2) * (ew.fo[i] - ef.fo[i]);
-    q.Sh[i] += C(2) * (ew.he[i] - ef.he[i]);
-    q.Dh[i] += C(2) * (ew.ho[i] - ef.ho[i]) - C(i < 2 ? 6.0 / 9.0 : 6.0 / 36.0) * en[i] * qn;
+    const int s = i >> 1;
+    const C e2 = ew.eu[i] * ew.eu[i];
+    q.S[i] += C(2) * (ew.A[s] + ew.B[s] * e2);
+    q.D[i] += C(2) * (ew.L[s] * ew.eu[i]);
+    q.Sh[i] += C(2) * (ew.HA[s] + ew.HB[s] * e2);
+    q.Dh[i] += C(2) * (ew.HL[s] * ew.eu[i]) - C(i < 2 ? 6.0 / 9.0 : 6.0 / 36.0) * en[i] * qn;
   }
   C v[NPOP];
   pair_collide<C, M & ~MODE_CORR, false>(kp, g.mu_law, q, w, C(0), C(0), v);
@@ -308,14 +316,6 @@ __device__ __forceinline__ void tile_ghost(const Grid& g, const S* src, S* __res
     dst[slot(g, a, dx - ex(a), dy - ey(a))] = Io<S>::from(v[a]);
     dst[slot(g, 9 + a, dx - ex(a), dy - ey(a))] = Io<S>::from(v[9 + a]);
   }
-}
-
-// -Q of the mirror ghost across a wall side: 2 rho u_w (theta_w - 1) - q.
-template <class C>
-__device__ __forceinline__ C mirror_q(const Grid& g, int side, int comp, C rho, C th, C q) {
-  const Phys<C>& k = phys<C>(g);
-  const C thw = g.bc[side] == BC_ISO ? k.thw[side] : th;
-  return C(2) * rho * k.uw[side][comp] * (thw - C(1)) - q;
 }
 
 template <class S, int M>
