@@ -1,14 +1,15 @@
 // Batched step: many independent grids of different sizes and physics modes
 // advance together.  One launch per time step covers every grid: a persistent
 // grid of blocks (one per resident slot) takes work items from a list -- each
-// item is the share of one block of the single-grid pulled-row kernel
-// (pr_block: 128 columns x `rows` rows of one grid) -- either round-robin or
+// item is the share of one block of the single-grid kernel (pair_block, or
+// pr_block for FP64: 128 columns x `rows` rows of one grid) -- either round-robin or
 // from an atomic counter.  Per-grid descriptors (buffers, TMA descriptors of
 // both buffers, step parity, steps left in the segment) live in device memory,
 // so a CUDA graph of k launches is captured once per k and replayed while the
 // host edits the descriptors between segments.
 #pragma once
 
+#include "lbm_pair.cuh"
 #include "lbm_step_pr.cuh"
 
 namespace lbm {
@@ -57,31 +58,39 @@ static_assert(bgk_index(BGK_MODES[0]) == 0 && bgk_index(BGK_MODES[3]) == 3 &&
                   bgk_index(BGK_MODES[5]) == 5 && bgk_index(BGK_MODES[7]) == 7,
               "mode slots follow BGK_MODES");
 
-// Ring depth (0: as the single-grid kernel) and resident blocks per SM that
-// the register budget of the batched kernel is sized for.
+// Block of the batched kernel: FP32 and 16-bit storage take the step over column
+// pairs (pair_block), FP64 the pulled-row step (pr_block); both own 128 columns
+// and issue their copies from the first thread of the helper warp.
 template <class S>
-__host__ __device__ constexpr int batch_depth() {
-  return 0;
-}
-template <class S>
-__host__ __device__ constexpr int batch_min_blocks() {
-  return sizeof(S) == 8 ? 3 : 4;
-}
+struct BatchGeom {
+  static constexpr bool pairs = sizeof(S) < 8;
+  static constexpr int threads = pairs ? PAIR_THREADS : PR_THREADS;
+  static constexpr int fetcher = pairs ? PAIR_COMPUTE : PR_COMPUTE;
+  static constexpr int min_blocks = pairs ? 5 : 3;
+  static constexpr size_t smem_bytes() {
+    if constexpr (pairs)
+      return PairGeom<S>::BYTES;
+    else
+      return PrGeom<S, 1, 0, 1>::smem_bytes();
+  }
+};
 template <class S, int M>
-__global__ void __launch_bounds__(PR_THREADS, (batch_min_blocks<S>()))
+__global__ void __launch_bounds__(BatchGeom<S>::threads, BatchGeom<S>::min_blocks)
     batch_step_kernel(const BatchGrid* __restrict__ grids, const WorkItem* __restrict__ items,
                       BatchCtl* ctl, int j) {
   constexpr int MS = mode_slot(M);
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ int s_item;
   __shared__ Grid s_grid;
-  constexpr int DD = batch_depth<S>();
-  pr_init<S, 1, DD>(smem);
+  if constexpr (BatchGeom<S>::pairs)
+    pair_init<S>(smem);
+  else
+    pr_init<S, 1>(smem);
   const int b0 = ctl->begin[MS], b1 = ctl->end[MS];
   const bool dyn = ctl->dynamic != 0;
   // helper lane 0 issues the copies; it also takes the items from the queue,
   // one ahead, so that the next item's first rows are staged early
-  const bool fetcher = threadIdx.x == PR_COMPUTE;
+  const bool fetcher = threadIdx.x == BatchGeom<S>::fetcher;
   int rr = b0 + blockIdx.x;  // round-robin cursor
   auto fetch = [&]() {       // next item of a grid that steps at j
     for (;;) {
@@ -127,8 +136,13 @@ __global__ void __launch_bounds__(PR_THREADS, (batch_min_blocks<S>()))
     __syncthreads();
     const int par = (int)((bg.t0 + j) & 1);
     int pre_out = 0;
-    const int st = pr_block<S, 1, M, DD, 1>(s_grid, &bg.maps[par], bg.buf[par], bg.buf[par ^ 1], w.x0,
-                                     w.y0, w.rows, smem, kbase, pre, next, &pre_out);
+    int st;
+    if constexpr (BatchGeom<S>::pairs)
+      st = pair_block<S, M>(s_grid, &bg.maps[par], bg.buf[par], bg.buf[par ^ 1], w.x0, w.y0,
+                            w.rows, smem, kbase, pre, next, &pre_out);
+    else
+      st = pr_block<S, 1, M, 0, 1>(s_grid, &bg.maps[par], bg.buf[par], bg.buf[par ^ 1], w.x0,
+                                   w.y0, w.rows, smem, kbase, pre, next, &pre_out);
     if (st) return;  // timeout recorded in the grid's status word
     kbase += pr_staged_rows(s_grid, w.y0, w.rows);
     // every thread passed the share's last barrier: s_item and s_grid are free

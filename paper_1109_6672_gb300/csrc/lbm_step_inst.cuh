@@ -101,7 +101,7 @@ template <class S, int M>
 cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j,
                       int blocks, cudaStream_t stream, int* occ) {
   static bool configured = false;
-  const size_t smem = PrGeom<S, 1, batch_depth<S>(), 1>::smem_bytes();
+  const size_t smem = BatchGeom<S>::smem_bytes();
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(batch_step_kernel<S, M>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -109,9 +109,10 @@ cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* c
     configured = true;
   }
   if (occ)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_step_kernel<S, M>, PR_THREADS,
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_step_kernel<S, M>,
+                                                         BatchGeom<S>::threads,
                                                          smem);
-  batch_step_kernel<S, M><<<blocks, PR_THREADS, smem, stream>>>(grids, items, ctl, j);
+  batch_step_kernel<S, M><<<blocks, BatchGeom<S>::threads, smem, stream>>>(grids, items, ctl, j);
   return cudaGetLastError();
 }
 
