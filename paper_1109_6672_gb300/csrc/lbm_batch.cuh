@@ -74,10 +74,12 @@ struct BatchGeom {
       return PrGeom<S, 1, 0, 1>::smem_bytes();
   }
 };
+// Step j of a segment; jc: the counter of the work queue (j, but for launches that
+// repeat a step to time it).
 template <class S, int M>
 __global__ void __launch_bounds__(BatchGeom<S>::threads, BatchGeom<S>::min_blocks)
     batch_step_kernel(const BatchGrid* __restrict__ grids, const WorkItem* __restrict__ items,
-                      BatchCtl* ctl, int j) {
+                      BatchCtl* ctl, int j, int jc) {
   constexpr int MS = mode_slot(M);
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ int s_item;
@@ -96,7 +98,7 @@ __global__ void __launch_bounds__(BatchGeom<S>::threads, BatchGeom<S>::min_block
     for (;;) {
       int it;
       if (dyn) {
-        it = b0 + atomicAdd(&ctl->counters[MS][j], 1);
+        it = b0 + atomicAdd(&ctl->counters[MS][jc], 1);
       } else {
         it = rr;
         rr += gridDim.x;
@@ -111,6 +113,10 @@ __global__ void __launch_bounds__(BatchGeom<S>::threads, BatchGeom<S>::min_block
     nxt = s_item < b1 ? fetch() : b1;
   }
   __syncthreads();
+  // what came before reads only what no step writes (and this step's own
+  // counter); from here on the previous step has to be complete
+  pdl_wait();
+  pdl_release();
   for (;;) {
     const int it = s_item;
     if (it >= b1) break;

@@ -4,6 +4,6 @@
 
 namespace lbm {
 template cudaError_t launch_batch_step<float>(const BatchGrid*, const WorkItem*, BatchCtl*,
-                                           int, int, int, cudaStream_t);
+                                           int, int, int, int, cudaStream_t, bool);
 template int occupancy_batch<float>(int);
 }  // namespace lbm

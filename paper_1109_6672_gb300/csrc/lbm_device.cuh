@@ -296,7 +296,8 @@ __device__ __forceinline__ void pull(const Grid& g, const S* __restrict__ src, i
   }
 }
 
-// The same, stored values as they are (Io::raw).
+// The same, stored values as they are (Io::raw), past L1 (the launches that use
+// it may start while the previous step still runs).
 template <class S>
 __device__ __forceinline__ void pull_raw(const Grid& g, const S* __restrict__ src, int x, int y,
                                          typename Io<S>::C d[NPOP]) {
@@ -304,7 +305,7 @@ __device__ __forceinline__ void pull_raw(const Grid& g, const S* __restrict__ sr
 #pragma unroll
   for (int a = 0; a < NPOP; ++a) {
     const int q = a % 9;
-    d[a] = Io<S>::raw(Io<S>::ld(p + (plane(a) - plane(0)) * g.pitch - ey(q) * g.rp - ex(q)));
+    d[a] = Io<S>::raw(__ldcg(p + (plane(a) - plane(0)) * g.pitch - ey(q) * g.rp - ex(q)));
   }
 }
 

@@ -44,10 +44,12 @@ struct WorkItem;
 struct BatchCtl;
 
 // One step of the batched kernel (lbm_batch.cuh) for the items of physics
-// mode `mode` over `blocks` persistent blocks, and its resident blocks per SM.
+// mode `mode` over `blocks` persistent blocks (pdl: the launch may start while the
+// kernel before it in the stream, the step before, still runs), and its
+// resident blocks per SM.
 template <class S>
 cudaError_t launch_batch_step(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j,
-                              int mode, int blocks, cudaStream_t stream);
+                              int jc, int mode, int blocks, cudaStream_t stream, bool pdl);
 template <class S>
 int occupancy_batch(int mode);
 

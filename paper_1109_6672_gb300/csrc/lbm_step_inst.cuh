@@ -98,8 +98,8 @@ cudaError_t launch_step_tma(const Grid& g, const CUtensorMap& map, int variant, 
 }
 
 template <class S, int M>
-cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j,
-                      int blocks, cudaStream_t stream, int* occ) {
+cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j, int jc,
+                      int blocks, cudaStream_t stream, bool pdl, int* occ) {
   static bool configured = false;
   const size_t smem = BatchGeom<S>::smem_bytes();
   if (!configured) {
@@ -112,28 +112,37 @@ cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* c
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_step_kernel<S, M>,
                                                          BatchGeom<S>::threads,
                                                          smem);
-  batch_step_kernel<S, M><<<blocks, BatchGeom<S>::threads, smem, stream>>>(grids, items, ctl, j);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(BatchGeom<S>::threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, batch_step_kernel<S, M>, grids, items, ctl, j, jc);
 }
 
 template <class S>
-cudaError_t batch_mode(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j,
-                       int mode, int blocks, cudaStream_t stream, int* occ) {
+cudaError_t batch_mode(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j, int jc,
+                       int mode, int blocks, cudaStream_t stream, bool pdl, int* occ) {
   return dispatch_mode<true>(mode, [&](auto m) {
-    return batch_one<S, decltype(m)::value>(grids, items, ctl, j, blocks, stream, occ);
+    return batch_one<S, decltype(m)::value>(grids, items, ctl, j, jc, blocks, stream, pdl, occ);
   });
 }
 
 template <class S>
 cudaError_t launch_batch_step(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j,
-                              int mode, int blocks, cudaStream_t stream) {
-  return batch_mode<S>(grids, items, ctl, j, mode, blocks, stream, nullptr);
+                              int jc, int mode, int blocks, cudaStream_t stream, bool pdl) {
+  return batch_mode<S>(grids, items, ctl, j, jc, mode, blocks, stream, pdl, nullptr);
 }
 
 template <class S>
 int occupancy_batch(int mode) {
   int occ = 0;
-  batch_mode<S>(nullptr, nullptr, nullptr, 0, mode, 1, nullptr, &occ);
+  batch_mode<S>(nullptr, nullptr, nullptr, 0, 0, mode, 1, nullptr, false, &occ);
   return occ;
 }
 
