@@ -100,7 +100,8 @@ typedef struct lbm3d_handle lbm3d_handle;
 int64_t lbm3d_state_bytes(const lbm3d_params* p);
 
 /* Validates *p and allocates the state and the staging of host transfers
- * (5 nx ny nz doubles) on the current device; binds the handle to
+ * (5 nx ny nz doubles; with walls also six values per node of a side) on the
+ * current device; binds the handle to
  * cuda_stream (NULL: the legacy default stream).  Errors: LBM_ERR_PARAM
  * (nx, ny or nz < 1, tau <= 0, R T0 != 1/3, b < 3, an unknown model,
  * precision or side kind, one side of an axis periodic and the other a
@@ -148,8 +149,8 @@ int64_t lbm3d_steps_done(const lbm3d_handle* h);
  * not depend on it beyond FP32 rounding): a block owns 32 x tile_rows nodes
  * of (x, y) and marches along z.  tile_rows = 8 or 16 (16 for LBM_P_FP32
  * only), with the halo ring on the tile's first threads; 0 = automatic
- * (LBM_P_FP64: 8 rows; LBM_P_FP32: 4 rows with halo warps, see
- * lbm3d_set_launch).  LBM_ERR_PARAM for other values. */
+ * (LBM_P_FP64: 32 x 8 or 16 x 16 nodes, whichever leaves fewer idle;
+ * LBM_P_FP32: 4 rows with halo warps, see lbm3d_set_launch).  LBM_ERR_PARAM for other values. */
 int lbm3d_set_tile(lbm3d_handle* h, int32_t tile_rows);
 
 /* Launch shape of the step kernel with the halo option (no counterpart in

@@ -27,8 +27,10 @@ struct lbm3d_handle {
   int tile_split = 0;  // separate halo warps asked for (tile != 0)
   int tile_rows = 8;   // tile rows in use
   int split = 0;       // separate halo warps in use
+  int lx = 5;          // log2 of the tile's columns
   double* staging = nullptr;  // 5 n doubles (host transfers), later 38 n (get_state)
   size_t staging_bytes = 0;
+  void* walls = nullptr;      // moments of the wall nodes between a step's two kernels
   double* partial = nullptr;  // reduction partials + result + flag
   std::string err;
 };
@@ -204,18 +206,19 @@ cudaError_t aux(lbm3d_handle* h, int what, void* buf, const double* const* in, d
                           h->stream);
 }
 
-// Launch shape: 32 x TY tiles of (x, y).  Automatic: FP64 8 rows; FP32 4
-// rows with separate halo warps (two 224-thread blocks per SM), which at
-// 256^3 ran at 11.1 GLUPS against 10.3 for 8 rows with the halo ring on the
-// tile's first threads (those threads pulled twice per plane while the rest
-// of the block waited), 9.2 for 8 rows with halo warps (one 352-thread block
-// per SM by registers) and 9.0 for 16 rows (one 512-thread block).  The z
-// range of a block is chosen so that the grid is about four waves of
-// resident blocks.
-size_t smem3(bool f64, int ty) {
-  if (f64) return step3d_smem<double, 8>();
-  return ty == 16 ? step3d_smem<float, 16>()
-                  : (ty == 4 ? step3d_smem<float, 4>() : step3d_smem<float, 8>());
+// Launch shape: tiles of (x, y), a z range of each per block.  Automatic: FP64 256
+// cells, 32 x 8 or 16 x 16; FP32 32 x 4 with separate halo warps and asynchronous
+// copies (two 224-thread blocks per SM), which steps 256^3 nodes in 1.16 ms against
+// 1.28 for 32 x 8 without, 1.30 for 32 x 8 with halo warps (one 352-thread block) and
+// 1.41 for 32 x 16 (one 512-thread block); 32 x 6 with halo warps took 1.34, and three
+// blocks of 32 x 4 at 80 registers 1.35 (both leave 28 KB of L1).  The z range (and the
+// FP64 tile) is the one with the fewest planes on the fullest slot: a block's first and
+// last plane only serve the differences, half a plane's work each in FP64, three
+// quarters in FP32, where they are read from memory.  Four waves of blocks instead took
+// 27.0 us a step for 64^3 FP32 nodes, against 23.0.
+size_t smem3(int ty, int split) {
+  if (split) return ty == 4 ? step3d_smem<float, 4, true>() : step3d_smem<float, 8, true>();
+  return ty == 16 ? step3d_smem<float, 16, false>() : step3d_smem<float, 8, false>();
 }
 int threads_of3(int ty, int split) {
   if (!split) return TX3 * ty;
@@ -226,23 +229,34 @@ void choose_launch(lbm3d_handle* h) {
   h->tile_rows = f64 ? 8 : (h->tile ? h->tile : 4);
   h->split = f64 ? 0 : (h->tile ? h->tile_split : 1);
   const int TYr = h->tile_rows;
-  const int tx = (h->p.nx + TX3 - 1) / TX3, ty = (h->p.ny + TYr - 1) / TYr;
-  cudaFuncAttributes a{};
-  const int mode = mode3_of(h->grid);
-  const cudaError_t e = f64 ? step3d_attributes_f64(mode, TYr, h->split, &a)
-                            : step3d_attributes_f32(mode, TYr, h->split, &a);
-  int per_sm = 1;
-  if (e == cudaSuccess && a.numRegs > 0)
-    per_sm = std::max(1, 65536 / (a.numRegs * threads_of3(TYr, h->split)));
-  // and by shared memory (the parked populations and the Q ring, plus the
-  // 1 KB the hardware reserves per block, of 228 KB per SM)
-  const size_t smem = smem3(f64, TYr);
-  per_sm = std::max(1, std::min(per_sm, (int)(233472 / (smem + 1024))));
+  int per_sm = 1;  // FP64: one block of 256 cells
+  if (!f64) {
+    cudaFuncAttributes a{};
+    const cudaError_t e = step3d_attributes_f32(mode3_of(h->grid), TYr, h->split, &a);
+    if (e == cudaSuccess && a.numRegs > 0)
+      per_sm = std::max(1, 65536 / (a.numRegs * threads_of3(TYr, h->split)));
+    // and by shared memory (the parked populations and the q ring, plus the
+    // 1 KB the hardware reserves per block, of 228 KB per SM)
+    per_sm = std::max(1, std::min(per_sm, (int)(233472 / (smem3(TYr, h->split) + 1024))));
+  }
   const long long resident = (long long)per_sm * std::max(1, h->num_sms);
-  const long long chunks =
-      std::max<long long>(1, std::min<long long>(h->p.nz, (4 * resident + tx * ty - 1) / (tx * ty)));
-  h->zrows = (int)((h->p.nz + chunks - 1) / chunks);
-  h->launch = dim3(tx, ty, (h->p.nz + h->zrows - 1) / h->zrows);
+  long long best = -1;
+  for (int lx = 5; lx >= (f64 && !h->tile ? 4 : 5); --lx) {
+    const int tx = (h->p.nx + (1 << lx) - 1) >> lx;
+    const int ty = (h->p.ny + (TX3 * TYr >> lx) - 1) / (TX3 * TYr >> lx);
+    for (int zr = 1; zr <= std::min(h->p.nz, 1024); ++zr) {
+      const int chunks = (h->p.nz + zr - 1) / zr;
+      if (chunks > 65535) continue;  // the grid's limit
+      const long long cost =
+          ((long long)tx * ty * chunks + resident - 1) / resident * (2 * zr + (f64 ? 1 : 3));
+      if (best < 0 || cost < best) {
+        best = cost;
+        h->lx = lx;
+        h->zrows = zr;
+        h->launch = dim3(tx, ty, chunks);
+      }
+    }
+  }
 }
 
 }  // namespace
@@ -273,7 +287,12 @@ int lbm3d_create(const lbm3d_params* p, void* stream, lbm3d_handle** out) {
   cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
   h->buf_bytes = buffer_bytes3(p);
   const size_t n = (size_t)p->nx * p->ny * p->nz;
+  fill_grid3(p, h->grid);
+  bool walled = false;
+  for (int s = 0; s < 6; ++s) walled |= h->grid.bc[s] != BC3_PERIODIC;
   if (cudaMalloc(&h->base, 2 * h->buf_bytes) != cudaSuccess ||
+      (walled && cudaMalloc(&h->walls, wall_values3(h->grid) *
+                                           (p->precision == LBM_P_FP64 ? 8 : 4)) != cudaSuccess) ||
       cudaMalloc(&h->partial, sizeof(double) * (5 * RED_BLOCKS3 + 8)) != cudaSuccess ||
       ensure_staging3(h, 5 * n * sizeof(double)) != LBM_OK) {
     cudaGetLastError();
@@ -286,7 +305,7 @@ int lbm3d_create(const lbm3d_params* p, void* stream, lbm3d_handle** out) {
     lbm3d_destroy(h);
     return fail3(nullptr, LBM_ERR_CUDA, std::string("memset: ") + cudaGetErrorString(e));
   }
-  fill_grid3(p, h->grid);
+  h->grid.wm = h->walls;
   choose_launch(h);
   *out = h;
   return LBM_OK;
@@ -335,9 +354,9 @@ int lbm3d_step(lbm3d_handle* h, int64_t n) {
     g.src = buf_ptr3(h, h->cur);
     g.dst = buf_ptr3(h, h->cur ^ 1);
     const cudaError_t e = h->p.precision == LBM_P_FP64
-                              ? launch_step3d_f64(g, h->launch, h->zrows, 8, 0, h->stream)
+                              ? launch_step3d_f64(g, h->launch, h->zrows, 8, 0, h->lx, h->stream)
                               : launch_step3d_f32(g, h->launch, h->zrows, h->tile_rows,
-                                                  h->split, h->stream);
+                                                  h->split, 5, h->stream);
     if (e != cudaSuccess) return cuda_fail3(h, e, "step kernel launch");
     h->cur ^= 1;
     ++h->steps;
@@ -446,6 +465,7 @@ void lbm3d_destroy(lbm3d_handle* h) {
   if (!h) return;
   if (h->stream || h->base) cudaStreamSynchronize(h->stream);
   if (h->base) cudaFree(h->base);
+  if (h->walls) cudaFree(h->walls);
   if (h->partial) cudaFree(h->partial);
   if (h->staging) cudaFree(h->staging);
   delete h;

@@ -2,9 +2,9 @@
 #include "lbm3d_inst.cuh"
 
 namespace lbm3 {
-cudaError_t launch_step3d_f64(const Grid3& g, dim3 grid, int zrows, int ty, int split,
+cudaError_t launch_step3d_f64(const Grid3& g, dim3 grid, int zrows, int ty, int split, int lx,
                               cudaStream_t st) {
-  return launch_step3d<double>(g, grid, zrows, ty, split, st);
+  return launch_step3d<double>(g, grid, zrows, ty, split, lx, st);
 }
 cudaError_t launch_aux3d_f64(int what, const Grid3& g, void* buf, const double* const* in,
                              double* const* out, double T0, double* pops, int* flag,

@@ -7,52 +7,86 @@
 namespace lbm3 {
 
 template <class S, int M, int TY, bool SPLIT>
-cudaError_t launch_tile3(const Grid3& g, dim3 grid, int zrows, cudaStream_t st) {
-  constexpr size_t SM = step3d_smem<S, TY>();
+constexpr auto step3d() {
+  if constexpr (SPLIT)
+    return step3d_async_kernel<S, M, TY>;
+  else
+    return step3d_kernel<S, M, TY>;
+}
+
+// The step, then the ghost slots of the walls, if there are any.
+template <class S, int M, int TY, bool SPLIT>
+cudaError_t launch_tile3(const Grid3& g, dim3 grid, int zrows, int lx, cudaStream_t st) {
+  constexpr size_t SM = step3d_smem<S, TY, SPLIT>();
   static bool attr_set = false;  // per process and instantiation (one device attribute)
   if (!attr_set) {
     const cudaError_t e = cudaFuncSetAttribute(
-        step3d_kernel<S, M, TY, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
+        step3d<S, M, TY, SPLIT>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  step3d_kernel<S, M, TY, SPLIT><<<grid, threads3<TY, SPLIT>(), SM, st>>>(g, zrows);
-  return cudaGetLastError();
+  if constexpr (SPLIT)
+    step3d_async_kernel<S, M, TY><<<grid, threads3<TY, true>(), SM, st>>>(g, zrows);
+  else
+    step3d_kernel<S, M, TY><<<grid, threads3<TY, false>(), SM, st>>>(g, zrows, lx);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  WallSides w{};
+  int sides = 0;
+  long long nodes = 0;
+  const long long n[3] = {(long long)g.ny * g.nz, (long long)g.nx * g.nz, (long long)g.nx * g.ny};
+  for (int s = 0; s < 6; ++s)
+    if (g.bc[s] != BC3_PERIODIC) {
+      w.side[sides++] = s;
+      nodes = n[s / 2] > nodes ? n[s / 2] : nodes;
+    }
+  if (!sides) return cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((nodes + WALL3_NODES - 1) / WALL3_NODES), sides);
+  cfg.blockDim = dim3(WALL3_NODES);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, walls3d_kernel<S, M>, g, w);
 }
 
-// Launch shapes (tile rows, separate halo warps): (8, no) for both
-// precisions; for FP32 storage also (16, no), (4, yes) and (8, yes).
+// Launch shapes (tile rows, separate halo warps): (8, no) for both precisions
+// (step3d_kernel); for FP32 storage also (16, no) and, with asynchronous copies
+// (step3d_async_kernel), (4, yes) and (8, yes).
 template <class S, int M>
-cudaError_t launch_mode3(const Grid3& g, dim3 grid, int zrows, int ty, int split,
+cudaError_t launch_mode3(const Grid3& g, dim3 grid, int zrows, int ty, int split, int lx,
                          cudaStream_t st) {
   if constexpr (sizeof(S) == 4) {
-    if (ty == 16) return launch_tile3<S, M, 16, false>(g, grid, zrows, st);
-    if (ty == 4 && split) return launch_tile3<S, M, 4, true>(g, grid, zrows, st);
-    if (ty == 8 && split) return launch_tile3<S, M, 8, true>(g, grid, zrows, st);
+    if (ty == 16) return launch_tile3<S, M, 16, false>(g, grid, zrows, lx, st);
+    if (ty == 4 && split) return launch_tile3<S, M, 4, true>(g, grid, zrows, lx, st);
+    if (ty == 8 && split) return launch_tile3<S, M, 8, true>(g, grid, zrows, lx, st);
   }
-  return launch_tile3<S, M, 8, false>(g, grid, zrows, st);
+  return launch_tile3<S, M, 8, false>(g, grid, zrows, lx, st);
 }
 
 template <class S>
-cudaError_t launch_step3d(const Grid3& g, dim3 grid, int zrows, int ty, int split,
+cudaError_t launch_step3d(const Grid3& g, dim3 grid, int zrows, int ty, int split, int lx,
                           cudaStream_t st) {
   switch (mode3_of(g)) {
     case M3_TOTAL | M3_ZFULL | M3_CORR:
-      return launch_mode3<S, M3_TOTAL | M3_ZFULL | M3_CORR>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_TOTAL | M3_ZFULL | M3_CORR>(g, grid, zrows, ty, split, lx, st);
     case M3_TOTAL | M3_ZFULL:
-      return launch_mode3<S, M3_TOTAL | M3_ZFULL>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_TOTAL | M3_ZFULL>(g, grid, zrows, ty, split, lx, st);
     case M3_TOTAL | M3_CORR:
-      return launch_mode3<S, M3_TOTAL | M3_CORR>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_TOTAL | M3_CORR>(g, grid, zrows, ty, split, lx, st);
     case M3_TOTAL:
-      return launch_mode3<S, M3_TOTAL>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_TOTAL>(g, grid, zrows, ty, split, lx, st);
     case M3_CORR:
-      return launch_mode3<S, M3_CORR>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_CORR>(g, grid, zrows, ty, split, lx, st);
     case M3_FORCE | M3_CORR:
-      return launch_mode3<S, M3_FORCE | M3_CORR>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_FORCE | M3_CORR>(g, grid, zrows, ty, split, lx, st);
     case M3_FORCE:
-      return launch_mode3<S, M3_FORCE>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, M3_FORCE>(g, grid, zrows, ty, split, lx, st);
     default:
-      return launch_mode3<S, 0>(g, grid, zrows, ty, split, st);
+      return launch_mode3<S, 0>(g, grid, zrows, ty, split, lx, st);
   }
 }
 
@@ -60,21 +94,21 @@ template <class S, int TY, bool SPLIT>
 cudaError_t attributes3d_tile(int mode, cudaFuncAttributes* a) {
   switch (mode) {
     case M3_TOTAL | M3_ZFULL | M3_CORR:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_TOTAL | M3_ZFULL | M3_CORR, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_TOTAL | M3_ZFULL | M3_CORR, TY, SPLIT>());
     case M3_TOTAL | M3_ZFULL:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_TOTAL | M3_ZFULL, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_TOTAL | M3_ZFULL, TY, SPLIT>());
     case M3_TOTAL | M3_CORR:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_TOTAL | M3_CORR, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_TOTAL | M3_CORR, TY, SPLIT>());
     case M3_TOTAL:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_TOTAL, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_TOTAL, TY, SPLIT>());
     case M3_CORR:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_CORR, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_CORR, TY, SPLIT>());
     case M3_FORCE | M3_CORR:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_FORCE | M3_CORR, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_FORCE | M3_CORR, TY, SPLIT>());
     case M3_FORCE:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, M3_FORCE, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, M3_FORCE, TY, SPLIT>());
     default:
-      return cudaFuncGetAttributes(a, step3d_kernel<S, 0, TY, SPLIT>);
+      return cudaFuncGetAttributes(a, step3d<S, 0, TY, SPLIT>());
   }
 }
 

@@ -20,10 +20,11 @@ inline int mode3_of(const Grid3& g) {
   return m;
 }
 
-// ty: tile rows; split: separate halo warps (launch_mode3 lists the shapes)
-cudaError_t launch_step3d_f64(const Grid3& g, dim3 grid, int zrows, int ty, int split,
+// ty: tile rows; split: separate halo warps (launch_mode3 lists the shapes); lx:
+// log2 of the tile's columns (FP64: 5, or 4 with 16 rows; FP32: 5)
+cudaError_t launch_step3d_f64(const Grid3& g, dim3 grid, int zrows, int ty, int split, int lx,
                               cudaStream_t st);
-cudaError_t launch_step3d_f32(const Grid3& g, dim3 grid, int zrows, int ty, int split,
+cudaError_t launch_step3d_f32(const Grid3& g, dim3 grid, int zrows, int ty, int split, int lx,
                               cudaStream_t st);
 cudaError_t launch_aux3d_f64(int what, const Grid3& g, void* buf, const double* const* in,
                              double* const* out, double T0, double* pops, int* flag,

@@ -70,11 +70,14 @@ __device__ __forceinline__ double rcp_(double v) {
   const double e = fma(-v, x, 1.0);
   return fma(x, fma(e, e, e), x);
 }
-__device__ __forceinline__ float rcp_(float v) { return __frcp_rn(v); }
 __device__ __forceinline__ float rcp_approx(float v) {
   float x;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(v));
   return x;
+}
+__device__ __forceinline__ float rcp_(float v) {
+  const float x = rcp_approx(v);
+  return fmaf(x, fmaf(v, -x, 1.0f), x);
 }
 __device__ __forceinline__ F2 rcp_(F2 v) {
   const F2 x(rcp_approx(v.v.x), rcp_approx(v.v.y));
