@@ -31,14 +31,14 @@ METRIC = "coupled f+h D2Q9 GLUPS and % HBM roofline; served p50/p99 latency"
 UNIT = "GLUPS"
 
 # DRAM bytes (read + write) of one step launch at 4096^2, from one ncu capture
-# at 2048^2 scaled by the node count (profiles/step_pr_*_2048_full.md), keyed
+# at 2048^2 scaled by the node count (profiles/step_pair_*_2048_full.md), keyed
 # by the hash of the kernel sources they were measured on; a changed kernel
 # reports null until it is captured again.
-KERNEL_SOURCES = ("lbm_device.cuh", "lbm_step_tma.cuh", "lbm_step_pr.cuh")
+KERNEL_SOURCES = ("lbm_device.cuh", "lbm_step_tma.cuh", "lbm_node.cuh", "lbm_pair.cuh")
 MEASURED_TRAFFIC = {
-    ("f35a03e90c75e143", "f32"): 2300.923904e6,
-    ("f35a03e90c75e143", "bf16"): 1091.465216e6,
-    ("f35a03e90c75e143", "f16"): 1096.441856e6,
+    ("9c7b130a10186ee2", "f32"): 2309.230592e6,
+    ("9c7b130a10186ee2", "bf16"): 1130.816512e6,
+    ("9c7b130a10186ee2", "f16"): 1131.144192e6,
 }
 
 
@@ -690,7 +690,7 @@ def run_ours(args, rank, world, local_rank):
                        "replicas": world},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "traffic": traffic, "peak_kind": peak_kind,
-                         "kernel": "step_pr_kernel", "algorithmic_bytes_per_launch": nodes * bpn,
+                         "kernel": "step_pair_kernel", "algorithmic_bytes_per_launch": nodes * bpn,
                          "traffic_note": "DRAM read+write bytes per launch from ncu at 2048^2, "
                                          "scaled x4 (node count); null if the kernel changed"},
             "cpu_baseline": cpu,
