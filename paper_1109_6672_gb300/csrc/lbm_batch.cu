@@ -144,8 +144,14 @@ int rows_of(const lbm_batch* b) {
   return b->rows > 0 ? b->rows : tma_default_rows(elem_bytes(b->precision));
 }
 
+void drop_graphs(lbm_batch* b) {
+  for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
+  b->graphs.clear();
+}
+
 // Work list: every (grid, strip, row block) of the active grids, largest grids
-// first so that the long items start early.
+// first so that the long items start early.  The launches of the cached graphs
+// hold the list's address, so they go when it grows.
 int rebuild_items(lbm_batch* b) {
   std::vector<int> order;
   for (int s = 0; s < (int)b->slots.size(); ++s)
@@ -178,6 +184,7 @@ int rebuild_items(lbm_batch* b) {
     end[ms] = (int)b->h_items.size();
   }
   if (b->h_items.size() > b->item_cap) {
+    drop_graphs(b);
     if (b->d_items) cudaFree(b->d_items);
     b->item_cap = std::max<size_t>(b->h_items.size() * 2, 1024);
     if (cudaMalloc(&b->d_items, b->item_cap * sizeof(WorkItem)) != cudaSuccess) {
@@ -354,11 +361,6 @@ int graph_for(lbm_batch* b, int64_t k, cudaGraphExec_t* out) {
   b->graphs[key] = exec;
   *out = exec;
   return LBM_OK;
-}
-
-void drop_graphs(lbm_batch* b) {
-  for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
-  b->graphs.clear();
 }
 
 int check_status(lbm_batch* b) {

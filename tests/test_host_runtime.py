@@ -1,0 +1,85 @@
+"""What the library's host code asks of the CUDA runtime, seen on the CPU: the calls run
+in a process of their own over a stand-in for the runtime (fake_cudart.cpp), which
+launches nothing but checks and records every launch."""
+import json
+import os
+import subprocess
+import sys
+from pathlib import Path
+
+import pytest
+
+from paper_1109_6672_gb300 import build
+
+ROOT = Path(__file__).resolve().parents[1]
+PROLOGUE = """
+import ctypes, json
+import numpy as np
+from paper_1109_6672_gb300 import inputs, lbm, lbm3d
+
+fake = ctypes.CDLL(None)
+fake.fake_graphs.restype = ctypes.c_longlong
+
+
+def counts():
+    a = (ctypes.c_longlong * 5)()
+    fake.fake_counts(a)
+    return dict(zip(("launches", "stale", "refused", "no_attr", "replayed"), a))
+
+
+def last():  # grid x, y, z, threads, dynamic shared memory of the last launch
+    a = (ctypes.c_longlong * 5)()
+    fake.fake_last(a)
+    return list(a)
+
+
+def rest(p):
+    shape = [p[k] for k in ("nz", "ny", "nx") if k in p]
+    one, zero = np.ones(shape), np.zeros(shape)
+    return [one] + [zero] * len(shape) + [one]
+
+
+def status(call):
+    try:
+        call()
+        return 0
+    except lbm.LbmError as e:
+        return e.status
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    """run(code) -> the JSON value that the code prints."""
+    build.build()
+    so = tmp_path_factory.mktemp("fake") / "fake_cudart.so"
+    include = Path(build.nvcc()).resolve().parents[1] / "include"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{include}",
+                    str(ROOT / "tests" / "fake_cudart.cpp"), "-o", str(so)], check=True)
+
+    def go(code):
+        env = dict(os.environ, LD_PRELOAD=str(so), PYTHONPATH=str(ROOT))
+        r = subprocess.run([sys.executable, "-c", PROLOGUE + code], env=env, capture_output=True,
+                           text=True, timeout=600)
+        assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
+        return json.loads(r.stdout)
+
+    return go
+
+
+def test_replayed_batch_graph_uses_the_current_work_list(run):
+    """A batch that outgrows its work list between two runs of the same length: the
+    second run replays no launch that holds the freed list."""
+    got = run("""
+fake.fake_pointers(1)
+b = lbm.Batch(lbm.LBM_P_FP32, 8, 1 << 28)
+b.set_schedule(1, 1)  # an item a row: 1024 are allocated at first
+p, f = inputs.cavity(n=300, precision=lbm.LBM_P_FP32)
+b.add(p, f, 100)
+b.run(10)
+for _ in range(3):
+    b.add(p, f, 100)
+b.run(10)
+print(json.dumps(counts()))
+""")
+    assert got["replayed"] == 20 and got["stale"] == 0
