@@ -21,16 +21,18 @@ constexpr int COST_NODE = 170, COST_HALO = 40;
 // time; 2540 instructions on the fullest SM) took 38 us a step, in 8 x 12 tiles
 // (five an SM; 2950) 33.7, in 32 x 4 tiles (four; 3200) 37.9; the 198^2 cavity
 // 24.6 in 16 x 6 (1770), 33.6 in 16 x 8 (2280).
-// rows > 0: that many rows per tile (as many as fit).
+// rows > 0: that many rows per tile (as many as fit the nodes and, with the
+// correction, the halo's two warps).  W = 1 always gives a tile.
 void tile_shape(int nx, int ny, bool corr, int sms, int rows, int* lw_out, int* rows_out) {
   long long best = -1;
   for (int lw = 5; lw >= 0; --lw) {
     const int W = 1 << lw;
     if (lw > 0 && W / 2 >= nx) continue;  // a narrower tile holds the row
-    const int most = std::min({TILE_MAX_NODES / W, 32, ny, rows > 0 ? rows : 32});
-    for (int R = rows > 0 ? most : 1; R <= most; ++R) {
+    const int most =
+        std::min({TILE_MAX_NODES / W, 32, ny, rows > 0 ? rows : 32,
+                  corr ? (TILE_MAX_THREADS - TILE_MAX_NODES) / 2 - W : 32});  // 2 W + 2 R
+    for (int R = rows > 0 ? std::max(most, 1) : 1; R <= most; ++R) {
       const int warps = (W * R + 31) / 32, halo = corr ? (2 * W + 2 * R + 31) / 32 : 0;
-      if (32 * halo > TILE_MAX_THREADS - TILE_MAX_NODES) continue;
       const long long blocks = (long long)((nx + W - 1) / W) * ((ny + R - 1) / R);
       const long long cost = (blocks + sms - 1) / sms * (warps * COST_NODE + halo * COST_HALO);
       if (best < 0 || cost < best) {

@@ -33,6 +33,7 @@ int device = 0;
 cudaError_t last_error = cudaSuccess;
 std::set<std::pair<const void*, int>> big_smem;  // kernels allowed > 48 KB, by device
 std::vector<long long> last;            // shape of the last launch
+int second[4];                          // and the first four words of its second argument
 struct Counts {
   long long launches, stale, refused, no_attr, replayed;
 } n;
@@ -59,6 +60,7 @@ cudaError_t launch(const void* f, dim3 grid, dim3 block, void** args, size_t sme
   Launch l{grid, block, smem, {nullptr, nullptr, nullptr}};
   if (ex && pointers)
     for (int i = 0; i < 3; ++i) l.ptr[i] = *static_cast<void**>(args[i]);
+  if (ex) std::memcpy(second, args[1], sizeof(second));
   last = {grid.x, grid.y, grid.z, block.x, (long long)smem};
   if (capturing) captured->nodes.push_back(l);
   return cudaSuccess;
@@ -73,6 +75,7 @@ void fake_pointers(int on) { pointers = on != 0; }
 void fake_fail_in(long long k) { fail_in = k; }
 void fake_device(int d) { device = d; }
 void fake_counts(long long* out) { std::memcpy(out, &n, sizeof(n)); }
+void fake_second(int* out) { std::memcpy(out, second, sizeof(second)); }
 long long fake_graphs() { return (long long)graphs.size(); }
 void fake_last(long long* out) { for (size_t i = 0; i < last.size(); ++i) out[i] = last[i]; }
 

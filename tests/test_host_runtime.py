@@ -83,3 +83,31 @@ b.run(10)
 print(json.dumps(counts()))
 """)
     assert got["replayed"] == 20 and got["stale"] == 0
+
+
+def test_every_tile_request_gets_tiles_that_cover_the_grid(run):
+    """FP64 grids from one column on, any requested height: a tile that fits its limits
+    (96 nodes, two halo warps with the correction) and tiles that cover the grid."""
+    got = run("""
+bad = []
+for nx in (1, 2, 3, 4, 9, 33, 70):
+    for ny in (1, 2, 31, 32, 33, 64, 100):
+        for corr in (0, 1):
+            p = inputs.base_params(nx, ny, correction=corr)
+            g = lbm.Lbm(p).init(*rest(p))
+            for rows in (0, 1, 2, 30, 31, 32, 33, 50, 96, 1000):
+                g.set_launch(0, rows).step(1)
+                a = (ctypes.c_int * 4)()
+                fake.fake_second(a)
+                lw, r, tx, ghosts = a
+                W, (blocks, _, _, threads, _) = 1 << lw, last()
+                halo = -(-(2 * W + 2 * r) // 32) if corr else 0
+                ok = (0 < r <= (rows or 32) and W * r <= 96 and halo <= 2 and tx == -(-nx // W)
+                      and blocks - ghosts == tx * -(-ny // r)
+                      and threads == 32 * (-(-W * r // 32) + halo))
+                if not ok:
+                    bad.append((nx, ny, corr, rows, lw, r))
+            g.close()
+print(json.dumps(bad))
+""")
+    assert got == []
