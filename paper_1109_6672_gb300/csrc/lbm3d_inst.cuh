@@ -41,16 +41,9 @@ cudaError_t launch_tile3(const Grid3& g, dim3 grid, int zrows, int lx, cudaStrea
       nodes = n[s / 2] > nodes ? n[s / 2] : nodes;
     }
   if (!sides) return cudaSuccess;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((nodes + WALL3_NODES - 1) / WALL3_NODES), sides);
-  cfg.blockDim = dim3(WALL3_NODES);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, walls3d_kernel<S, M>, g, w);
+  return lbm::launch_ex(walls3d_kernel<S, M>,
+                        dim3((unsigned)((nodes + WALL3_NODES - 1) / WALL3_NODES), sides),
+                        WALL3_NODES, 0, st, true, g, w);
 }
 
 // Launch shapes (tile rows, separate halo warps): (8, no) for both precisions

@@ -25,6 +25,26 @@ __device__ __forceinline__ void pdl_release() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Launch, with pdl as a programmatic dependent of the launch before it in the
+// stream.  A refused launch leaves no pending error behind for the next call.
+template <class... P, class... A>
+cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
+                      cudaStream_t stream, bool pdl, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 // Two FP32 values, one per node: add, mul and fma are single packed
 // instructions (add/mul/fma.rn.f32x2), which issue at half the instructions
 // per node of scalar FP32 (the packed fma reached the same 128 fma per SM and

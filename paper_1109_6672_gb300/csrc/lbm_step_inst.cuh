@@ -35,17 +35,7 @@ cudaError_t launch_one(const Grid& g, const CUtensorMap& map, int rows, dim3 gri
     configured = true;
   }
   if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, threads, smem);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = NPT == 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, g, map, rows);
+  return launch_ex(kernel, grid, threads, smem, stream, NPT == 1, g, map, rows);
 }
 
 // Calls fn(std::integral_constant<int, M>{}) for the kernel of physics mode
@@ -112,17 +102,8 @@ cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* c
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_step_kernel<S, M>,
                                                          BatchGeom<S>::threads,
                                                          smem);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(BatchGeom<S>::threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, batch_step_kernel<S, M>, grids, items, ctl, j, jc);
+  return launch_ex(batch_step_kernel<S, M>, dim3(blocks), BatchGeom<S>::threads, smem, stream, pdl,
+                   grids, items, ctl, j, jc);
 }
 
 template <class S>

@@ -74,17 +74,10 @@ cudaError_t launch_step_tile(const Grid& g, int lw, int rows, cudaStream_t strea
   }
   const int warps = (W * rows + 31) / 32;
   const int halo = g.correction ? (2 * W + 2 * rows + 31) / 32 : 0;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ta.ghost_blocks + ta.tx * ((g.ny + rows - 1) / rows));
-  cfg.blockDim = dim3(32 * (warps + halo));
-  cfg.stream = stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
+  const dim3 grid(ta.ghost_blocks + ta.tx * ((g.ny + rows - 1) / rows));
   return dispatch_mode<true>(mode_of(g), [&](auto m) {
-    return cudaLaunchKernelEx(&cfg, step_tile_kernel<double, decltype(m)::value>, g, ta);
+    return launch_ex(step_tile_kernel<double, decltype(m)::value>, grid, 32 * (warps + halo), 0,
+                     stream, true, g, ta);
   });
 }
 

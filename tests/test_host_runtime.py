@@ -111,3 +111,19 @@ for nx in (1, 2, 3, 4, 9, 33, 70):
 print(json.dumps(bad))
 """)
     assert got == []
+
+
+@pytest.mark.parametrize("step", ["lbm.Lbm(inputs.base_params(9, 9))",
+                                  "lbm.Lbm(inputs.base_params(9, 9, precision=1))",
+                                  "lbm3d.Lbm3d(inputs.base_params3d(5, 5, 5, bc_z=[1, 1], "
+                                  "T_wall_z=[1.0, 1.0]))"])
+def test_a_refused_step_leaves_no_error_for_the_next_call(run, step):
+    got = run(f"""
+g, h = {step}, {step}
+f = rest(dict(zip(("nx", "ny", "nz"), g.shape[::-1])))
+g.init(*f)
+fake.fake_fail_in(ctypes.c_longlong(1 if len(f) == 5 else 0))  # 3-D: the walls' launch
+print(json.dumps([status(lambda: g.step(1)), status(lambda: h.init(*f)),
+                  status(lambda: h.step(1))]))
+""")
+    assert got == [-3, 0, 0]
