@@ -368,10 +368,10 @@ int lbm_set_steps_done(lbm_handle* h, int64_t t);
  * 128 columns per block; for FP64 storage tiles of nodes, one per thread.
  * 2: TMA staging with 256 columns per block (two per thread); 64..256, a
  * multiple of 32: the register-pull kernel, each block owning variant - 2
- * columns.  rows_per_block >= 1, or 0 for the default (6 rows for FP32
- * storage, 12 for 16-bit storage, for the TMA kernel; chosen from the grid for
- * tiles; about one wave of blocks for the register-pull kernel); tiles take as
- * many of the rows asked for as fit one.  rows_per_block (and the block width of the
+ * columns.  rows_per_block >= 1, or 0 for the default (chosen from the grid; 6
+ * rows for the TMA kernel on large FP32 grids); tiles take as many of the rows
+ * asked for as fit one, the other kernels at least ny / 65535 (the launch's limit
+ * of row blocks).  rows_per_block (and the block width of the
  * register-pull kernel) never changes a bit of the result; different variants
  * agree to rounding (different FMA contraction).  Variant 2 is built for the
  * BGK collision with constant relaxation times only (LBM_ERR_PARAM with

@@ -655,7 +655,8 @@ int step_rows(lbm_handle* h) {
   }
   if (h->rows <= 0 && h->auto_rows == 0)
     h->auto_rows = h->variant >= 64 ? auto_rows(h, h->variant) : tma_rows(h, h->variant);
-  return h->rows > 0 ? h->rows : h->auto_rows;
+  // the row blocks are the grid's y extent, 65535 at most
+  return std::max(h->rows > 0 ? h->rows : h->auto_rows, (h->p.ny + 65534) / 65535);
 }
 
 // Enqueue n steps on `stream` (the step kernel, then the second pass of the

@@ -127,3 +127,19 @@ print(json.dumps([status(lambda: g.step(1)), status(lambda: h.init(*f)),
                   status(lambda: h.step(1))]))
 """)
     assert got == [-3, 0, 0]
+
+
+def test_tall_grids_stay_within_the_launch_limits(run):
+    """A launch has at most 65535 blocks along y; grids have up to 2^20 rows."""
+    got = run("""
+out = []
+for precision in range(4):
+    p = inputs.base_params(4, 400000, precision=precision)
+    g = lbm.Lbm(p).init(*rest(p))
+    for variant, rows in ((0, 0), (0, 1), (2, 0), (2, 1), (128, 0), (128, 1)):
+        g.set_launch(variant, rows)
+        out.append(status(lambda: g.step(1)))
+    g.close()
+print(json.dumps([out, counts()["refused"]]))
+""")
+    assert got == [[0] * 24, 0]
