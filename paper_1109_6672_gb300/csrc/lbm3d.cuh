@@ -642,7 +642,14 @@ __host__ __device__ constexpr int step3d_min_blocks() {
   return sizeof(S) == 8 ? 1 : (SPLIT ? (TY == 4 ? 2 : 1) : (TY == 8 ? 2 : 1));
 }
 
-// Geometry of a block of the step kernels: its tile and z range, a cell's place.
+// First node of a block's tile (2^lx x TY cells): blockIdx.x counts the tiles of
+// (x, y), x first (along y alone a launch would end at 65535).
+__device__ __forceinline__ void tile_origin3(int nx, int lx, int TY, int& x0, int& y0) {
+  const int n = (nx + (1 << lx) - 1) >> lx, row = (int)blockIdx.x / n;
+  x0 = ((int)blockIdx.x - row * n) << lx;
+  y0 = row * TY;
+}
+
 // q at plane r - 1 around cell `cell` and at planes r - 2 and r, as differences
 // dq[k][j] = q_j(x + e_k) - q_j(x - e_k); across a wall Eq. 50 takes the mirror
 // ghost (mirror_q3).  qc: the ring's plane r - 1; q2, q1, q0: q at planes r - 2 .. r.
@@ -732,7 +739,9 @@ __global__ void __launch_bounds__(threads3<TY, false>(), (step3d_min_blocks<S, T
   const int t = threadIdx.x;
   const int tx = t & (TXr - 1), ty = t >> lx;
   const int nx = g.nx, ny = g.ny, nz = g.nz;
-  const int x0 = blockIdx.x * TXr, y0 = blockIdx.y * TYr, z0 = blockIdx.z * zrows;
+  int x0, y0;
+  tile_origin3(nx, lx, TYr, x0, y0);
+  const int z0 = blockIdx.z * zrows;
   if (z0 >= nz) return;
   const int z1 = min(z0 + zrows, nz);
   const S* src = static_cast<const S*>(g.src);
@@ -836,7 +845,9 @@ __global__ void __launch_bounds__(threads3<TY, true>(), (step3d_min_blocks<S, TY
 
   const int t = threadIdx.x;
   const int nx = g.nx, ny = g.ny, nz = g.nz;
-  const int x0 = blockIdx.x * TX3, y0 = blockIdx.y * TY, z0 = blockIdx.z * zrows;
+  int x0, y0;
+  tile_origin3(nx, 5, TY, x0, y0);
+  const int z0 = blockIdx.z * zrows;
   if (z0 >= nz) return;
   const int z1 = min(z0 + zrows, nz);
   const S* src = static_cast<const S*>(g.src);

@@ -253,7 +253,7 @@ void choose_launch(lbm3d_handle* h) {
         best = cost;
         h->lx = lx;
         h->zrows = zr;
-        h->launch = dim3(tx, ty, chunks);
+        h->launch = dim3((unsigned)tx * ty, 1, chunks);
       }
     }
   }

@@ -143,3 +143,18 @@ for precision in range(4):
 print(json.dumps([out, counts()["refused"]]))
 """)
     assert got == [[0] * 24, 0]
+
+
+def test_3d_grids_wide_along_y_stay_within_the_launch_limits(run):
+    got = run("""
+out = []
+for precision, shapes in ((0, ((0, 0), (8, 0))), (1, ((0, 0), (8, 0), (16, 0), (8, 1)))):
+    p = inputs.base_params3d(2, 1100000, 1, precision=precision)
+    g = lbm3d.Lbm3d(p).init(*rest(p))
+    for shape in shapes:
+        g.set_launch(*shape)
+        out.append(status(lambda: g.step(1)))
+    g.close()
+print(json.dumps([out, counts()["refused"]]))
+""")
+    assert got == [[0] * 6, 0]
