@@ -18,18 +18,14 @@ constexpr auto step3d() {
 template <class S, int M, int TY, bool SPLIT>
 cudaError_t launch_tile3(const Grid3& g, dim3 grid, int zrows, int lx, cudaStream_t st) {
   constexpr size_t SM = step3d_smem<S, TY, SPLIT>();
-  static bool attr_set = false;  // per process and instantiation (one device attribute)
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        step3d<S, M, TY, SPLIT>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<unsigned long long> allowed{0};
+  cudaError_t e = lbm::allow_smem((const void*)step3d<S, M, TY, SPLIT>(), (int)SM, allowed);
+  if (e != cudaSuccess) return e;
   if constexpr (SPLIT)
     step3d_async_kernel<S, M, TY><<<grid, threads3<TY, true>(), SM, st>>>(g, zrows);
   else
     step3d_kernel<S, M, TY><<<grid, threads3<TY, false>(), SM, st>>>(g, zrows, lx);
-  const cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   WallSides w{};
   int sides = 0;

@@ -224,22 +224,24 @@ int upload_grids(lbm_batch* b) {
              : bfail(b, LBM_ERR_CUDA, "descriptor upload failed");
 }
 
+// Blocks of the persistent launch of a physics mode (0: no block fits an SM).
 int blocks_of(lbm_batch* b, int mode) {
   int& occ = b->occ_mode[mode_slot(mode)];
   if (!occ) {
     by_precision(b->precision, [&](auto* tag) {
       using S = std::remove_pointer_t<decltype(tag)>;
-      occ = std::max(1, occupancy_batch<S>(mode));
+      occ = std::max(0, occupancy_batch<S>(mode));
       return cudaSuccess;
     });
   }
-  return std::max(1, occ * b->num_sms);
+  return occ * std::max(1, b->num_sms);
 }
 
 // Step j of the group of physics mode `mode`, with work-queue counter jc.
 cudaError_t launch_mode_step(lbm_batch* b, int mode, int j, int jc, cudaStream_t stream,
                              bool pdl) {
   const int blocks = blocks_of(b, mode);
+  if (blocks == 0) return cudaErrorLaunchOutOfResources;
   return by_precision(b->precision, [&](auto* tag) {
     using S = std::remove_pointer_t<decltype(tag)>;
     return launch_batch_step<S>(b->d_grids, b->d_items, b->d_ctl, j, jc, mode, blocks, stream, pdl);

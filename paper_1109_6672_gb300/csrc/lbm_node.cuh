@@ -14,6 +14,8 @@
 // C is double, float, or F2 (two nodes at once in packed FP32 instructions).
 #pragma once
 
+#include <atomic>
+
 #include "lbm_step_tma.cuh"
 
 namespace lbm {
@@ -42,6 +44,22 @@ cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, int threads, size_t smem,
   cfg.numAttrs = pdl ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
+// Allows a kernel `bytes` of dynamic shared memory.  The attribute belongs to a
+// device: `done` (one per kernel) has a bit for each that has it.
+inline cudaError_t allow_smem(const void* kernel, int bytes, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0;  // (beyond: every time)
+  if (e == cudaSuccess && (done.load(std::memory_order_acquire) & bit)) return e;
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess)
+    done.fetch_or(bit, std::memory_order_release);
+  else
+    cudaGetLastError();
   return e;
 }
 

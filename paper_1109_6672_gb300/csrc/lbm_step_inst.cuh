@@ -28,12 +28,9 @@ cudaError_t launch_one(const Grid& g, const CUtensorMap& map, int rows, dim3 gri
     threads = PR_THREADS;
     smem = (int)PrGeom<S, NPT>::smem_bytes();
   }
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<unsigned long long> allowed{0};
+  const cudaError_t e = allow_smem((const void*)kernel, smem, allowed);
+  if (e != cudaSuccess) return e;
   if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, threads, smem);
   return launch_ex(kernel, grid, threads, smem, stream, NPT == 1, g, map, rows);
 }
@@ -90,14 +87,10 @@ cudaError_t launch_step_tma(const Grid& g, const CUtensorMap& map, int variant, 
 template <class S, int M>
 cudaError_t batch_one(const BatchGrid* grids, const WorkItem* items, BatchCtl* ctl, int j, int jc,
                       int blocks, cudaStream_t stream, bool pdl, int* occ) {
-  static bool configured = false;
+  static std::atomic<unsigned long long> allowed{0};
   const size_t smem = BatchGeom<S>::smem_bytes();
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(batch_step_kernel<S, M>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  const cudaError_t e = allow_smem((const void*)batch_step_kernel<S, M>, (int)smem, allowed);
+  if (e != cudaSuccess) return e;
   if (occ)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, batch_step_kernel<S, M>,
                                                          BatchGeom<S>::threads,

@@ -158,3 +158,24 @@ for precision, shapes in ((0, ((0, 0), (8, 0))), (1, ((0, 0), (8, 0), (16, 0), (
 print(json.dumps([out, counts()["refused"]]))
 """)
     assert got == [[0] * 6, 0]
+
+
+def test_each_device_gets_the_kernels_shared_memory(run):
+    """The limit of dynamic shared memory is raised per kernel and device."""
+    got = run("""
+out = []
+for device in (0, 1, 0):
+    fake.fake_device(device)
+    for precision in (0, 1):
+        p = inputs.base_params(64, 64, precision=precision)
+        b = lbm.Batch(precision, 1, 1 << 26)
+        b.add(p, rest(p), 9)
+        out.append(status(lambda: b.run(1)))
+        g = lbm.Lbm(p).set_launch(2, 0).init(*rest(p))
+        out.append(status(lambda: g.step(1)))
+        p = inputs.base_params3d(8, 8, 8, precision=precision)
+        g = lbm3d.Lbm3d(p).init(*rest(p))
+        out.append(status(lambda: g.step(1)))
+print(json.dumps([out, counts()["no_attr"]]))
+""")
+    assert got == [[0] * 18, 0]
