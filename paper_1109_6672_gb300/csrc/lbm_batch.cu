@@ -330,16 +330,18 @@ int build_graph(lbm_batch* b, int64_t k, bool advance, cudaGraphExec_t* out) {
   Branches br;
   if (!b->has_fix && br.make(b->stream, (int)b->modes.size()) != cudaSuccess)
     return bfail(b, LBM_ERR_CUDA, "stream creation failed");
-  cudaGraph_t graph;
+  cudaGraph_t graph = nullptr;
   if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
     return bfail(b, LBM_ERR_CUDA, "stream capture failed to start");
   const size_t counter_bytes = sizeof(int) * BATCH_MODE_SLOTS * BATCH_MAX_SEG;
   cudaError_t e = cudaMemsetAsync(counters_of(b), 0, counter_bytes, b->stream);
   if (e == cudaSuccess) e = capture_steps(b, k, advance, br);
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &graph);
-  if (e != cudaSuccess || e2 != cudaSuccess)
+  if (e != cudaSuccess || e2 != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
     return bfail(b, LBM_ERR_CUDA, std::string("graph capture failed: ") +
                                       cudaGetErrorString(e != cudaSuccess ? e : e2));
+  }
   e = cudaGraphInstantiate(out, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, "graph instantiation failed");

@@ -179,3 +179,15 @@ for device in (0, 1, 0):
 print(json.dumps([out, counts()["no_attr"]]))
 """)
     assert got == [[0] * 18, 0]
+
+
+def test_a_failed_capture_leaves_no_graph_behind(run):
+    got = run("""
+p = inputs.base_params(64, 64, precision=1)
+b = lbm.Batch(1, 2, 1 << 26)
+b.add(p, rest(p), 9)
+fake.fake_fail_in(ctypes.c_longlong(1))
+print(json.dumps([status(lambda: b.run(3)), fake.fake_graphs(), status(lambda: b.run(3)),
+                  fake.fake_graphs()]))
+""")
+    assert got == [-3, 0, 0, 0]
