@@ -657,11 +657,12 @@ int lbm_batch_remove(lbm_batch* b, int32_t slot) {
 
 // Time one step of the current grids (without advancing them: the step reads
 // the current buffers and writes the other ones, which the next real step
-// overwrites) for each candidate schedule, `reps` times in a graph such as
-// lbm_batch_run() replays; keep the fastest.
+// overwrites) for each candidate schedule, at least `reps` times in graphs such as
+// lbm_batch_run() replays (of 256 steps at most: longer ones take longer to
+// instantiate than they add to the time's precision); keep the fastest.
 int lbm_batch_autotune(lbm_batch* b, int32_t reps, int64_t out_best[3]) {
   if (!b || reps < 1) return LBM_ERR_PARAM;
-  reps = std::min(reps, BATCH_MAX_SEG);  // counters of the work queue
+  const int64_t replays = ((int64_t)reps + 255) / 256, per = (reps + replays - 1) / replays;
   const int cand_rows[] = {4, 6, 8, 12, 16, 24};
   const int cand_dyn[] = {1, 0};
   float best = 1e30f;
@@ -685,12 +686,13 @@ int lbm_batch_autotune(lbm_batch* b, int32_t reps, int64_t out_best[3]) {
       b->dynamic = dyn;
       if ((rc = rebuild_items(b))) break;
       cudaGraphExec_t exec;
-      if ((rc = build_graph(b, reps, false, &exec))) break;
+      if ((rc = build_graph(b, per, false, &exec))) break;
       cudaError_t e = cudaGraphUpload(exec, b->stream);
       if (e == cudaSuccess && !warm) e = cudaGraphLaunch(exec, b->stream);
       warm = true;
       cudaEventRecord(e0, b->stream);
-      if (e == cudaSuccess) e = cudaGraphLaunch(exec, b->stream);
+      for (int64_t r = 0; r < replays && e == cudaSuccess; ++r)
+        e = cudaGraphLaunch(exec, b->stream);
       cudaEventRecord(e1, b->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       cudaGraphExecDestroy(exec);
@@ -719,7 +721,7 @@ int lbm_batch_autotune(lbm_batch* b, int32_t reps, int64_t out_best[3]) {
   if (out_best) {
     out_best[0] = best_rows;
     out_best[1] = best_dyn;
-    out_best[2] = (int64_t)std::llround(1e3 * best / reps);  // microseconds per step
+    out_best[2] = (int64_t)std::llround(1e3 * best / (replays * per));  // microseconds per step
   }
   return LBM_OK;
 }

@@ -191,3 +191,16 @@ print(json.dumps([status(lambda: b.run(3)), fake.fake_graphs(), status(lambda: b
                   fake.fake_graphs()]))
 """)
     assert got == [-3, 0, 0, 0]
+
+
+@pytest.mark.parametrize("reps", [1, 20, 257, 5000])
+def test_autotune_times_the_launches_asked_for(run, reps):
+    """12 candidates (6 heights, 2 ways to hand out items), each at least `reps` times."""
+    got = run(f"""
+p = inputs.base_params(64, 64, precision=1)
+b = lbm.Batch(1, 2, 1 << 26)
+b.add(p, rest(p), 9)
+b.autotune({reps})
+print(json.dumps(counts()["replayed"]))
+""")
+    assert 12 * reps <= got <= 13 * (reps + reps // 256 + 1)
