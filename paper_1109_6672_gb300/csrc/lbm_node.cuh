@@ -139,6 +139,14 @@ __device__ __forceinline__ float pow_(float v, float n) { return powf(v, n); }
 __device__ __forceinline__ F2 pow_(F2 v, F2 n) {
   return F2(powf(v.v.x, n.v.x), powf(v.v.y, n.v.y));
 }
+// min(v, a number whose square is far from overflow); NaN stays NaN.
+__device__ __forceinline__ double cap_(double v) { return v > 1e100 ? 1e100 : v; }
+__device__ __forceinline__ float cap_(float v) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "f"(1e15f));
+  return r;
+}
+__device__ __forceinline__ F2 cap_(F2 v) { return F2(cap_(v.v.x), cap_(v.v.y)); }
 
 // A node's populations as pairs: rest, sums, differences, of f and of h.
 template <class C>
@@ -231,7 +239,9 @@ __device__ __forceinline__ C mirror_q(const Grid& g, int side, int comp, C rho, 
 // (rho theta), tau_h = tau_f r, over one common reciprocal.  Sutherland:
 // L = theta^(3/2) (1 + s) / (theta + s), so with X = rho (theta + s) and
 // Y = 2 tau_f0 (1 + s) sqrt(theta), w_f = 2 X / (X + Y), w_h = 2 X / (X + r Y);
-// power law: X = rho theta, Y = 2 tau_f0 theta^n.  kz: w_h - w_f, or for MRT
+// power law: X = rho theta, Y = 2 tau_f0 theta^n.  Y is capped where w is zero to
+// rounding, so that neither an overflowing theta^n nor the product of the two
+// denominators turns it into NaN.  kz: w_h - w_f, or for MRT
 // (1 - w_h/2)(1/r - 1) w_f (Eq. 47 with tau_f + 1/2 = 1/w_f).
 template <class C, int M>
 __device__ __forceinline__ void pair_rates(const Phys<typename Scalar<C>::T>& k, int mu_law, C rho,
@@ -250,6 +260,7 @@ __device__ __forceinline__ void pair_rates(const Phys<typename Scalar<C>::T>& k,
       X = rho * (th + C(k.mu_s));
       Y = C(2 * k.tau_f0 * (1 + k.mu_s)) * sqrt_(th);
     }
+    Y = cap_(Y);
     const C a = X + Y, b = fma_(C(k.tau_ratio), Y, X);
     const C t = (X + X) * rcp_(a * b);
     wf = t * b;
