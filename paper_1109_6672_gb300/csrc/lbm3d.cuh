@@ -31,10 +31,11 @@
 //
 // Kernel: a block owns a tile of (x, y) and marches along z over its z range.
 // For each plane it first computes the moments (and q = -Q) of the tile plus a
-// one-node halo ring (wrapped periodically) into a 4-plane ring of q in shared
+// one-node halo ring (wrapped periodically) into a 3-plane ring of q in shared
 // memory, then collides the plane below, whose own moments the thread kept in
 // registers and whose pulled populations it parked in shared memory (a
-// per-thread column, two planes deep, so no barrier guards it).  Each side of the
+// per-thread column, two planes deep (three with asynchronous copies), so no
+// barrier guards it).  Each side of the
 // box is periodic or a halfway wall.
 #pragma once
 

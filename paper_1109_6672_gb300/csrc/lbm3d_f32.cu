@@ -12,6 +12,9 @@ cudaError_t launch_aux3d_f32(int what, const Grid3& g, void* buf, const double* 
   return launch_aux3d<float>(what, g, buf, in, out, T0, pops, flag, partial, blocks, st);
 }
 cudaError_t step3d_attributes_f32(int mode, int ty, int split, cudaFuncAttributes* a) {
-  return attributes3d<float>(mode, ty, split, a);
+  if (ty == 16) return attributes3d_tile<float, 16, false>(mode, a);
+  if (ty == 4 && split) return attributes3d_tile<float, 4, true>(mode, a);
+  if (ty == 8 && split) return attributes3d_tile<float, 8, true>(mode, a);
+  return attributes3d_tile<float, 8, false>(mode, a);
 }
 }  // namespace lbm3

@@ -11,7 +11,4 @@ cudaError_t launch_aux3d_f64(int what, const Grid3& g, void* buf, const double* 
                              double* partial, int blocks, cudaStream_t st) {
   return launch_aux3d<double>(what, g, buf, in, out, T0, pops, flag, partial, blocks, st);
 }
-cudaError_t step3d_attributes_f64(int mode, int ty, int split, cudaFuncAttributes* a) {
-  return attributes3d<double>(mode, ty, split, a);
-}
 }  // namespace lbm3

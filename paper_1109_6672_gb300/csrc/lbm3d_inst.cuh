@@ -102,16 +102,6 @@ cudaError_t attributes3d_tile(int mode, cudaFuncAttributes* a) {
 }
 
 template <class S>
-cudaError_t attributes3d(int mode, int ty, int split, cudaFuncAttributes* a) {
-  if constexpr (sizeof(S) == 4) {
-    if (ty == 16) return attributes3d_tile<S, 16, false>(mode, a);
-    if (ty == 4 && split) return attributes3d_tile<S, 4, true>(mode, a);
-    if (ty == 8 && split) return attributes3d_tile<S, 8, true>(mode, a);
-  }
-  return attributes3d_tile<S, 8, false>(mode, a);
-}
-
-template <class S>
 cudaError_t launch_aux3d(int what, const Grid3& g, void* buf, const double* const* in,
                          double* const* out, double T0, double* pops, int* flag, double* partial,
                          int blocks, cudaStream_t st) {

@@ -32,8 +32,7 @@ cudaError_t launch_aux3d_f64(int what, const Grid3& g, void* buf, const double* 
 cudaError_t launch_aux3d_f32(int what, const Grid3& g, void* buf, const double* const* in,
                              double* const* out, double T0, double* pops, int* flag,
                              double* partial, int blocks, cudaStream_t st);
-// step kernel attributes (registers, for the resident-block count)
-cudaError_t step3d_attributes_f64(int mode, int ty, int split, cudaFuncAttributes* attr);
+// attributes of an FP32 step kernel (registers, for the resident-block count)
 cudaError_t step3d_attributes_f32(int mode, int ty, int split, cudaFuncAttributes* attr);
 
 enum { AUX3_INIT = 0, AUX3_EXPORT = 1, AUX3_CONSERVED = 2 };

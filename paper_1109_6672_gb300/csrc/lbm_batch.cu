@@ -271,15 +271,6 @@ int* counters_of(lbm_batch* b) {
   return reinterpret_cast<int*>(reinterpret_cast<char*>(b->d_ctl) + offsetof(BatchCtl, counters));
 }
 
-// Captures k steps (advance) or step 0 k times on the batch's stream.  The groups of different physics modes
-// hold different grids, so their steps do not wait for one another: each group's
-// steps form a branch of the graph of its own, launch after launch with
-// programmatic dependent launch (a step's blocks set themselves up while the
-// last ones of the step before finish).  Open sides and walls of non-equilibrium
-// extrapolation are fixed up for all groups at once after every step; with one
-// of those present the groups take their steps one after another.
-// (28 cavities and 20 channels, us a step in one chain and in two branches: FP32
-// 97.1 and 86.7, BF16 105.1 and 95.2; 5 and 7 small ones, FP32: 21.8 and 13.2.)
 // Streams and events of the branches, made before the capture starts (branch 0
 // is the batch's stream).
 struct Branches {
@@ -304,6 +295,15 @@ struct Branches {
   }
 };
 
+// Captures k steps (advance) or step 0 k times on the batch's stream.  The groups of
+// different physics modes hold different grids, so their steps do not wait for one
+// another: each group's steps form a branch of the graph of its own, launch after
+// launch with programmatic dependent launch (a step's blocks set themselves up while
+// the last ones of the step before finish).  Open sides and walls of non-equilibrium
+// extrapolation are fixed up for all groups at once after every step; with one
+// of those present the groups take their steps one after another.
+// (28 cavities and 20 channels, us a step in one chain and in two branches: FP32
+// 97.1 and 86.7, BF16 105.1 and 95.2; 5 and 7 small ones, FP32: 21.8 and 13.2.)
 cudaError_t capture_steps(lbm_batch* b, int64_t k, bool advance, const Branches& br) {
   cudaError_t e = cudaSuccess;
   if (b->has_fix) {

@@ -1,7 +1,7 @@
 // Batched step: many independent grids of different sizes and physics modes
-// advance together.  One launch per time step covers every grid: a persistent
-// grid of blocks (one per resident slot) takes work items from a list -- each
-// item is the share of one block of the single-grid kernel (pair_block, or
+// advance together.  One launch per time step and physics mode covers every grid of
+// that mode: a persistent grid of blocks (one per resident slot) takes work items
+// from a list -- each item is the share of one block of the single-grid kernel (pair_block, or
 // pr_block for FP64: 128 columns x `rows` rows of one grid) -- either round-robin or
 // from an atomic counter.  Per-grid descriptors (buffers, TMA descriptors of
 // both buffers, step parity, steps left in the segment) live in device memory,

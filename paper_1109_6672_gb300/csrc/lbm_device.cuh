@@ -233,15 +233,19 @@ struct Io<__nv_bfloat16> {
 // neither on the launch shape nor on the other grids of a batch.
 constexpr unsigned SR_SEED = 0x2545F491u;
 
-__device__ __forceinline__ unsigned sr_hash(const Grid& g, int x, int y) {
-  unsigned h = ((unsigned)x * 0x9E3779B1u) ^ ((unsigned)y * 0x85EBCA77u) ^ (g.t * 0xC2B2AE3Du) ^
-               SR_SEED;
+// Hash of node (x, y); ht: sr_step of the step.
+__device__ __forceinline__ unsigned sr_step(unsigned t) { return (t * 0xC2B2AE3Du) ^ SR_SEED; }
+__device__ __forceinline__ unsigned sr_node(int x, int y, unsigned ht) {
+  unsigned h = ((unsigned)x * 0x9E3779B1u) ^ ((unsigned)y * 0x85EBCA77u) ^ ht;
   h ^= h >> 16;  // 32-bit integer finaliser (xor-shift-multiply)
   h *= 0x7FEB352Du;
   h ^= h >> 15;
   h *= 0x846CA68Bu;
   h ^= h >> 16;
   return h;
+}
+__device__ __forceinline__ unsigned sr_hash(const Grid& g, int x, int y) {
+  return sr_node(x, y, sr_step(g.t));
 }
 
 // Random words of a node: the linear congruential sequence
@@ -421,56 +425,6 @@ __device__ __forceinline__ void equilibria_es(C rho, C ux, C uy, C th, C Es, boo
     const C pb = C(-3) * usq - th;  // bracket of h^eq at e = 0: -3u^2 + th(-2)/2
     heq[0] = total ? Es * feq[0] + wgt<C>(0) * p * pb : Es * feq[0];
   }
-}
-
-// Equilibria of deviation storage as deviations from the rest equilibria
-// (rho = 1, u = 0, theta = 1, Es = b/6): fd_a = f^eq_a - w_a and
-// hd_a = h^eq_a - href_a from drho = rho - 1, dth = theta - 1 and
-// dEs = Es - b/6, so that only small quantities are rounded:
-//   f^eq_a - w_a = w_a [drho + rho (even_a - 1 + odd_a)],
-//   h^eq_a - href_a = Es (f^eq_a - w_a) + dEs w_a
-//                     + w_a [p (9 eu^2 - 3 u^2 +- 3 eu) + (p th - 1/3)(3 e^2 - 2)/2]
-// (the last line for the total-energy model; p th - 1/3 = (drho + rho dth
-// (2 + dth))/3).  The rest populations are the remainders of the sums
-// sum fd = drho and sum hd = sdh (the sum of the node's h deviations, since
-// rho Es = sum href + sdh), as in equilibria_es.
-template <class C>
-__device__ __forceinline__ void equilibria_dev(C drho, C ux, C uy, C dth, C dEs, C b6, bool total,
-                                               C sdh, C fd[9], C hd[9]) {
-  const C rho = C(1) + drho;
-  const C Es = b6 + dEs;
-  const C usq = ux * ux + uy * uy;
-  const C em1 = C(-1.5) * usq + C(0.5) * dth;  // even part - 1 without 9/2 eu^2: axis
-  const C em2 = C(-1.5) * usq + C(2) * dth;    // diagonal
-  const C lin1 = C(3) - C(1.5) * dth, lin2 = C(3) * (C(1) + dth);
-  const C p = rho * (C(1) + dth) * (C(1) / C(3));
-  const C pt = (drho + rho * dth * (C(2) + dth)) * (C(1) / C(3));  // p th - 1/3
-  const C hu = C(-3) * usq;
-  const C eus[4] = {ux, uy, ux + uy, uy - ux};  // e.u for a = 1, 2, 5, 6
-  const int ia[4] = {1, 2, 5, 6};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int a = ia[k], o = opp(a);
-    const C eu = eus[k];
-    const C w = wgt<C>(a);
-    const C evenm = (k < 2 ? em1 : em2) + C(4.5) * eu * eu;
-    const C odd = (k < 2 ? lin1 : lin2) * eu;
-    fd[a] = w * (drho + rho * (evenm + odd));
-    fd[o] = w * (drho + rho * (evenm - odd));
-    if (total) {
-      const C he = p * (hu + C(9) * eu * eu) + (k < 2 ? C(0.5) : C(2)) * pt;
-      const C ho = p * C(3) * eu;
-      hd[a] = Es * fd[a] + w * (dEs + he + ho);
-      hd[o] = Es * fd[o] + w * (dEs + he - ho);
-    } else {
-      hd[a] = Es * fd[a] + w * dEs;
-      hd[o] = Es * fd[o] + w * dEs;
-    }
-  }
-  const C sf = ((fd[1] + fd[2]) + (fd[3] + fd[4])) + ((fd[5] + fd[6]) + (fd[7] + fd[8]));
-  const C sh = ((hd[1] + hd[2]) + (hd[3] + hd[4])) + ((hd[5] + hd[6]) + (hd[7] + hd[8]));
-  fd[0] = drho - sf;
-  hd[0] = sdh - sh;
 }
 
 // The same from theta alone (Es from b / 6).

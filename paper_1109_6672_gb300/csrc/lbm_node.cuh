@@ -274,7 +274,7 @@ __device__ __forceinline__ void pair_rates(const Phys<typename Scalar<C>::T>& k,
 
 // Equilibria per pair, f^eq_a = fe + fo, f^eq_o = fe - fo (Eq. 18a), likewise
 // h^eq (Eq. 18b or the Eq. 38 form), as deviations from the rest equilibria for
-// deviation storage (the terms of equilibria_dev).  Per shell s (0: the axis
+// deviation storage.  Per shell s (0: the axis
 // pairs, 1: the diagonals) they are linear in e.u and its square,
 //   fe = A + B (e.u)^2, fo = L e.u, he = HA + HB (e.u)^2, ho = HL e.u:
 //   f^eq = w rho [base + 9/2 eu^2 +- lin eu],

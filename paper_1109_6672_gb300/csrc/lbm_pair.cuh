@@ -468,15 +468,7 @@ __device__ __forceinline__ int pair_columns(const Grid& g, S* __restrict__ dst, 
   const int xwall = (has1 && c == 0 && wall_l ? 1 : 0) | (c == nx - 1 && wall_r ? 2 : 0) |
                     (c + 1 == nx - 1 && wall_r ? 4 : 0);
   const bool xl = x0 == 0, xr = nx - 1 < x0 + PAIR_COLS;  // the block holds the side's column
-  const unsigned ht = (g.t * 0xC2B2AE3Du) ^ SR_SEED;
-  auto hash = [&](int x, int y) {  // sr_hash
-    unsigned h = ((unsigned)x * 0x9E3779B1u) ^ ((unsigned)y * 0x85EBCA77u) ^ ht;
-    h ^= h >> 16;
-    h *= 0x7FEB352Du;
-    h ^= h >> 15;
-    h *= 0x846CA68Bu;
-    return h ^ (h >> 16);
-  };
+  const unsigned ht = sr_step(g.t);
   // The y-edge rows' values wait in local memory (a thread's own) for the end of
   // the loop.
   constexpr int NKEEP = 28;
@@ -552,7 +544,7 @@ __device__ __forceinline__ int pair_columns(const Grid& g, S* __restrict__ dst, 
       S* p = dst + (long long)(ro + 1) * g.rp + XOFF + c;
       typename IO::W w[NPOP];
       if constexpr (Io<S>::sr) {
-        unsigned ra = hash(c, ro), rb = hash(c + 1, ro);
+        unsigned ra = sr_node(c, ro, ht), rb = sr_node(c + 1, ro, ht);
 #pragma unroll
         for (int a = 0; a < NPOP; a += 2) {
           // a node's word j rounds populations 2j (high half) and 2j + 1

@@ -49,17 +49,6 @@ struct TileArgs {
   double fin[3], hin[3];  // the inlet's populations 1, 5, 8 of this step
 };
 
-// Pull of node (x, y) past L1.
-template <class S>
-__device__ __forceinline__ void pull_cg(const Grid& g, const S* src, int x, int y, S d[NPOP]) {
-  const S* p = src + slot(g, 0, x, y);
-#pragma unroll
-  for (int a = 0; a < NPOP; ++a) {
-    const int q = a % 9;
-    d[a] = __ldcg(p + (plane(a) - plane(0)) * g.pitch - ey(q) * g.rp - ex(q));
-  }
-}
-
 // h^eq of direction A at (rho, u, theta) with the specific energy es, and f^eq.
 template <class C, int A>
 __device__ __forceinline__ void eq_at(bool total, C rho, C ux, C uy, C th, C es, C& f, C& h) {
@@ -241,7 +230,7 @@ __device__ __forceinline__ void tile_ghost(const Grid& g, const S* src, S* __res
   C d[NPOP], qx, qy;
   Pairs<C> q;
   Mom<C> m;
-  pull_cg<S>(g, src, fx, fy, d);
+  pull_raw<S>(g, src, fx, fy, d);
   to_pairs(d, q);
   pair_moments<C, M, false>(kp, q, m, qx, qy);
   Mom<C> w;  // the wall node's state
@@ -254,7 +243,7 @@ __device__ __forceinline__ void tile_ghost(const Grid& g, const S* src, S* __res
     C d2[NPOP];
     Pairs<C> q2;
     Mom<C> m2;
-    pull_cg<S>(g, src, fx - nxo, fy - nyo, d2);
+    pull_raw<S>(g, src, fx - nxo, fy - nyo, d2);
     to_pairs(d2, q2);
     pair_moments<C, M, false>(kp, q2, m2, qx, qy);
     w.th = fmax((C(4) * m.th - m2.th) * C(1.0 / 3.0), C(0.5) * m.th);
@@ -387,7 +376,7 @@ __global__ void __launch_bounds__(TILE_MAX_THREADS, 3)
   C qx = 0, qy = 0;
   if (what) {
     C d[NPOP];
-    pull_cg<S>(g, src, x, y, d);
+    pull_raw<S>(g, src, x, y, d);
     to_pairs(d, q);
     pair_moments<C, M, false>(k, q, m, qx, qy);
   }
