@@ -484,7 +484,10 @@ int create_impl(const lbm_params* p, void* stream, void* ext, int64_t ext_bytes,
 int block_cols(int variant) { return variant >= 64 ? variant - 2 : tma_cols(variant); }
 
 // Rows per block of the TMA kernels.  Large FP32 grids keep the default (6 rows:
-// many waves of short blocks, which HBM likes); a grid that needs fewer than 3
+// many waves of short blocks, which HBM likes), or one row less in the pair step from
+// 8 waves on (us a step with 6 and 5 rows: 4096^2 cavity 361.5 and 353.0, box 361.1
+// and 350.8; 2048^2 95.9 and 94.8; but 1700^2, 6 waves, 69.1 and 71.8, and 1024^2, 3
+// waves with 5 rows, 27.6 and 30.4); a grid that needs fewer than 3
 // waves of blocks at the default, and 16-bit storage on any grid, takes the row
 // count that minimises waves x (rows + 2) (the 2: a block's fixed cost of staging
 // its halo rows and starting up, in rows).
@@ -500,7 +503,8 @@ int tma_rows(const lbm_handle* h, int variant) {
   const long long slots = (long long)std::max(occ, 1) * std::max(1, h->num_sms);
   auto waves = [&](int r) { return ((long long)bx * ((h->p.ny + r - 1) / r) + slots - 1) / slots; };
   const bool large = waves(r0) >= 3;
-  if (large && elem_size(h->p.precision) != 2) return r0;
+  if (large && elem_size(h->p.precision) != 2)
+    return variant == TMA_PR_1 && waves(r0) >= 8 ? r0 - 1 : r0;
   int best = r0;
   long long cost = waves(r0) * (r0 + 2);
   for (int r = large ? 8 : 2; r <= std::min(h->p.ny, large ? 32 : 64); ++r) {
