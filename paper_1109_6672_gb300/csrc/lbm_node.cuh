@@ -353,14 +353,15 @@ __device__ __forceinline__ void pair_shells(const Phys<typename Scalar<C>::T>& k
 // C' = C_a (Eq. 49) + F_a.  With a = -dx / 24 and b = -dy / 24, C_a / 2 is
 // a - 2 b on the pair (1, 3), b - 2 a on (2, 4) and a + b on the diagonals
 // (the rest population follows from the conserved sum).
+// HEQ: at a wall node, v[19..26] take h^eq of the moving directions for the wall rules.
 // n = (f - f^eq) + C'/2 has no mass and no momentum; in it
 //   f* = f^eq + C'/2 + (1 - w_f) n          (BGK),
 //   f* = f^eq + C'/2 + M^-1 (1 - S) M n     (MRT),
 // and Eq. 36's coupling is kz Z n.
-template <class C, int M, bool DEV, int K = 1>
+template <class C, int M, bool DEV, int K = 1, bool HEQ = false>
 __device__ __forceinline__ void pair_collide(const Phys<typename Scalar<C>::T>& k, int mu_law,
-                                             const Pairs<C>& q, const Mom<C>& m, C dx, C dy,
-                                             C v[NPOP]) {
+                                             const Pairs<C>& q, const Mom<C>& m, C dx, C dy, C* v,
+                                             bool wall = false) {
   using MD = Mode<M>;
   using T = typename Scalar<C>::T;
   constexpr int A[4] = {1, 2, 5, 6};
@@ -412,6 +413,12 @@ __device__ __forceinline__ void pair_collide(const Phys<typename Scalar<C>::T>& 
     bE[i] = cf ? fe + c[i] : fe;
     bO[i] = gf ? fo + g : fo;
     const C he = fma_(e.HB[s], e2, e.HA[s]), ho = e.HL[s] * e.eu[i];
+    if constexpr (HEQ) {
+      if (wall) {
+        v[18 + a] = he + ho;
+        v[18 + o] = he - ho;
+      }
+    }
     // h* = h^eq + (1 - w_h)(h - h^eq)
     C hE = fma_(wh1, fma_(C(-2.0), he, q.Sh[i]), he);
     C hO = fma_(wh1, fma_(C(-2.0), ho, q.Dh[i]), ho);

@@ -209,6 +209,11 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
   using SM = PrSmem<S, NPT, DD, XD>;
   constexpr bool DEV = Io<S>::dev;  // moments carried as deviations (pair_moments)
   constexpr int K = Io<S>::scale;   // factor of the stored values
+  // h^eq of wall nodes comes out of the update in variant 2 with FP64 storage, where
+  // forming it again costs its edge warps about 60 FP64 operations in series (256^2
+  // box 56.2 -> 49.9 us a step, cavity 58.6 -> 55.0); FP64 batches spill with it, and
+  // with 16-bit storage it gains nothing
+  constexpr bool HEQ = sizeof(C) == 8 && XD == 0;
   constexpr int D = G::D, TWC = G::TWC;
   constexpr unsigned long long WAIT_NS = 2000000000ull;  // 2 s
   S* ring = SM::ring(smem);
@@ -380,7 +385,9 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
         m.es = pes[i];
         m.sh = pq.h0 + ((pq.Sh[0] + pq.Sh[1]) + (pq.Sh[2] + pq.Sh[3]));
         C v[27];
-        pair_collide<C, M, DEV, K>(phys<C>(g), g.mu_law, pq, m, qxr - qxl, qyu - qyd, v);
+        const bool wall = (c == 0 && wall_l) || (c == nx - 1 && wall_r) || (ro == 0 && wall_b) ||
+                          (ro == ny - 1 && wall_t);
+        pair_collide<C, M, DEV, K, HEQ>(phys<C>(g), g.mu_law, pq, m, qxr - qxl, qyu - qyd, v, wall);
         pr_store<S>(g, prow + c, pitch, c, ro, v);
         // ghost-slot writes (from absolute values): x edges inline (one
         // thread of a warp), the edge rows (every thread of the row) through
@@ -391,7 +398,7 @@ __device__ __forceinline__ int pr_block(const Grid& g, const CUtensorMap* map, c
 #pragma unroll
             for (int a = 0; a < 18; ++a) v[a] = v[a] * C(1.0 / K) + pref<S>(g, a);
           }
-          {  // h^eq with the node's own specific energy, for the wall rules
+          if constexpr (!HEQ) {  // h^eq with the node's own specific energy, for the wall rules
             C fq[9];
             equilibria_es<C>(rho_n, pux[i], puy[i], th_n,
                              DEV ? phys<C>(g).b6 + pes[i] : pes[i], Mode<M>::total, fq, v + 18);
