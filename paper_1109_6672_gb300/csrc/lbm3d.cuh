@@ -850,6 +850,12 @@ __global__ void __launch_bounds__(threads3<TY, true>(), (step3d_min_blocks<S, TY
   tile_origin3(nx, 5, TY, x0, y0);
   const int z0 = blockIdx.z * zrows;
   if (z0 >= nz) return;
+  // The walls' blocks may start (they wait for the whole step): with short z ranges, whose
+  // launch is what the step lasts, at once (us a step of walled ducts, released here, with
+  // the last plane, and before the walls had a launch of their own: 16^3 8.5, 10.3, 10.3;
+  // 32^3 10.3, 11.6, 10.3), else with the last plane, where they do not hold up the
+  // loads (128^3 released at once 190, with the last plane 180).
+  if (zrows <= 2) lbm::pdl_release();
   const int z1 = min(z0 + zrows, nz);
   const S* src = static_cast<const S*>(g.src);
   const Phys3<C>& ph = phys3<C>(g);
@@ -909,7 +915,7 @@ __global__ void __launch_bounds__(threads3<TY, true>(), (step3d_min_blocks<S, TY
       asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
-      lbm::pdl_release();
+      if (zrows > 2) lbm::pdl_release();
     }
     Mom3<C> cm = pm;
     if (interior) {
