@@ -96,14 +96,14 @@ typedef struct lbm3d_handle lbm3d_handle;
 
 /* Bytes of device memory of the two population buffers of a grid:
  * 2 (nz + 2)(ny + 2) 38 pitch elements, pitch = the smallest multiple of 32
- * >= nx + 33.  Negative LBM_ERR_* for invalid parameters. */
+ * >= nx + 33 (what lbm3d_create allocates besides is listed there).  Negative
+ * LBM_ERR_* for invalid parameters. */
 int64_t lbm3d_state_bytes(const lbm3d_params* p);
 
 /* Validates *p and allocates the state and the staging of host transfers
- * (5 nx ny nz doubles; with walls also six values per node of a side) on the
- * current device; binds the handle to
- * cuda_stream (NULL: the legacy default stream).  Errors: LBM_ERR_PARAM
- * (nx, ny or nz < 1, tau <= 0, R T0 != 1/3, b < 3, an unknown model,
+ * (5 nx ny nz doubles; with walls also 12 (ny nz + nx nz + nx ny) values of the
+ * storage's type) on the current device; binds the handle to cuda_stream (NULL:
+ * the legacy default stream).  Errors: LBM_ERR_PARAM (nx, ny or nz < 1, tau <= 0, R T0 != 1/3, b < 3, an unknown model,
  * precision or side kind, one side of an axis periodic and the other a
  * wall, a non-finite wall velocity, an isothermal wall's temperature <= 0,
  * a non-finite g or g != 0 with total energy, 2^31 nodes or more),
@@ -150,7 +150,8 @@ int64_t lbm3d_steps_done(const lbm3d_handle* h);
  * of (x, y) and marches along z.  tile_rows = 8 or 16 (16 for LBM_P_FP32
  * only), with the halo ring on the tile's first threads; 0 = automatic
  * (LBM_P_FP64: 32 x 8 or 16 x 16 nodes, whichever leaves fewer idle;
- * LBM_P_FP32: 4 rows with halo warps, see lbm3d_set_launch).  LBM_ERR_PARAM for other values. */
+ * LBM_P_FP32: 4 rows with halo warps, see lbm3d_set_launch).  LBM_ERR_PARAM for
+ * other values. */
 int lbm3d_set_tile(lbm3d_handle* h, int32_t tile_rows);
 
 /* Launch shape of the step kernel with the halo option (no counterpart in

@@ -823,9 +823,9 @@ __global__ void __launch_bounds__(threads3<TY, false>(), (step3d_min_blocks<S, T
 // shared memory (4-byte asynchronous copies, a thread its own) while planes r and
 // r - 1 are worked on, and warps of their own for the halo cells, which hold the next
 // plane's values in registers: FP32 storage.  Two blocks are resident; what bounds it
-// is the latency of the eight colliding warps' arithmetic (44 % of the issue slots used,
-// 57 % of the memory's rate), not the loads, which the copies hide.  256^3 nodes:
-// 1.44 ms a step with synchronous loads and the faces in the step, 1.16 now (5.1 GB, 0.73
+// is the latency of the eight colliding warps' arithmetic (at 128^3 44 % of the issue slots
+// used, 52 % of the memory's rate), not the loads, which the copies hide.  256^3 nodes:
+// 1.44 ms a step with synchronous loads and the faces in the step, 1.15 now (5.1 GB, 0.77
 // at the measured copy rate); 64^3 nodes 45.5 -> 23.0 us, a walled 101 x 87 x 65 duct
 // 90.8 -> 68.5.
 __device__ __forceinline__ void copy_async4(void* s, const void* p) {

@@ -9,10 +9,10 @@
 //    nodes an instruction;
 //  - stores are one 8-byte (FP32) or 4-byte (16-bit) word per population, and a
 //    16-bit conversion rounds both nodes' values of a population at once,
-// and a node takes 322 and 403.  us a step, before -> after: 1024^2 cavity BF16
-// 39.3 -> 29.4, 3001 x 2003 box FP16 248 -> 189, 512^2 cavity FP32 14.0 -> 9.6,
-// 1733 x 1021 MRT channel with a power-law viscosity FP32 80.9 -> 64.0; the
-// 4096^2 FP32 box, at 0.95 of the copy bandwidth, stays where it was.
+// and a node takes 331 (in blocks of 5 rows) and 390.  us a step (without reads of the fields), before ->
+// after: 1024^2 cavity BF16 37.0 -> 26.7, 3001 x 2003 box FP16 169.6 -> 134.0, 512^2
+// cavity FP32 13.2 -> 8.9, 1733 x 1021 MRT channel with a power-law viscosity FP32
+// 71.5 -> 54.8, 4096^2 box FP32 373.2 -> 350.8 (at the measured copy rate).
 // FP16 storage holds 256 x the deviation; the update runs on the scaled values
 // (every term is linear in them), which saves the scalings of loads and stores.
 //
@@ -23,12 +23,14 @@
 // forms q_x of the two columns beside the strip; one barrier a row publishes q_x
 // and frees the slot of row r - 1.
 //
-// Registers decide: the L1 left beside the rings is small, so anything spilled
-// goes to L2 (a version that kept the populations of the held row in registers
+// Registers decide: the L1 left beside the rings is small, so most of what is
+// spilled goes to L2 (a version that kept the populations of the held row in registers
 // spilled about 100 bytes a row and took 1.3 to 2 times as long).  So a row is
 // read from its slot twice, for q and for the collision, its moments are formed
 // again, the two roles have loops of their own, and nothing but the update itself
-// is in the row loop.  (Without a helper, each warp on its own with 64 columns and
+// is in the row loop.  At 128 registers FP32 storage spills nothing; 16-bit storage,
+// whose 18 packed results and random words are live together, 8 to 44 bytes (28 in the
+// cavity's mode).  (Without a helper, each warp on its own with 64 columns and
 // 12 to 16 warps an SM, the halo columns cost every warp a pass of its own: 376
 // and 488 instructions a node, 1024^2 BF16 31.1 us, 3001 x 2003 FP16 206.)
 //
