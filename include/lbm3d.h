@@ -103,7 +103,8 @@ int64_t lbm3d_state_bytes(const lbm3d_params* p);
 /* Validates *p and allocates the state and the staging of host transfers
  * (5 nx ny nz doubles; with walls also 12 (ny nz + nx nz + nx ny) values of the
  * storage's type) on the current device; binds the handle to cuda_stream (NULL:
- * the legacy default stream).  Errors: LBM_ERR_PARAM (nx, ny or nz < 1, tau <= 0, R T0 != 1/3, b < 3, an unknown model,
+ * the legacy default stream).  Errors: LBM_ERR_PARAM
+ * (nx, ny or nz < 1, tau <= 0, R T0 != 1/3, b < 3, an unknown model,
  * precision or side kind, one side of an axis periodic and the other a
  * wall, a non-finite wall velocity, an isothermal wall's temperature <= 0,
  * a non-finite g or g != 0 with total energy, 2^31 nodes or more),
